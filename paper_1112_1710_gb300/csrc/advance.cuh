@@ -192,11 +192,12 @@ template <> struct VecIO<double> {
 };
 
 // Stores the face state pw (primitives, xyz order) of the axis-d face in its
-// rotated frame.
+// rotated frame (d need not be a compile-time constant).
 template <typename R>
 __device__ __forceinline__ void store_face_state(R* g, int64_t sn, int64_t x, int d, const R (&pw)[8]) {
-  const int t1 = (d + 1) % 3, t2 = (d + 2) % 3;
-  const R v[7] = {pw[0], pw[1 + d], pw[1 + t1], pw[1 + t2], pw[4], pw[5 + t1], pw[5 + t2]};
+  auto pick = [d](R a, R b, R c) { return d == 0 ? a : (d == 1 ? b : c); };
+  const R v[7] = {pw[0], pick(pw[1], pw[2], pw[3]), pick(pw[2], pw[3], pw[1]), pick(pw[3], pw[1], pw[2]), pw[4],
+                  pick(pw[6], pw[7], pw[5]), pick(pw[7], pw[5], pw[6])};
   VecIO<R>::store7(g, sn, x, v);
 }
 
@@ -259,9 +260,9 @@ __global__ void __launch_bounds__(kThreads) k_prim(const DPatch* __restrict__ P,
     R u[8];
 #pragma unroll
     for (int q = 0; q < 5; ++q) u[q] = ((const R*)p.U[q])[x];
-    u[5] = R(0.5) * (((const R*)p.B[0])[x] + ((const R*)p.B[0])[x + 1]);
-    u[6] = R(0.5) * (((const R*)p.B[1])[x] + ((const R*)p.B[1])[x + p.s1]);
-    u[7] = R(0.5) * (((const R*)p.B[2])[x] + ((const R*)p.B[2])[x + p.s2]);
+    u[5] = Tr<R>::half(((const R*)p.B[0])[x] + ((const R*)p.B[0])[x + 1]);
+    u[6] = Tr<R>::half(((const R*)p.B[1])[x] + ((const R*)p.B[1])[x + p.s1]);
+    u[7] = Tr<R>::half(((const R*)p.B[2])[x] + ((const R*)p.B[2])[x + p.s2]);
     R w[8];
     cons2prim(u, sc.gm1, w);
     if constexpr (Cfl) {
@@ -273,7 +274,7 @@ __global__ void __launch_bounds__(kThreads) k_prim(const DPatch* __restrict__ P,
         for (int d = 0; d < 3; ++d) {
           const int t1 = (d + 1) % 3, t2 = (d + 2) % 3;
           R cf = fast_speed(w[0], w[4], w[5 + d], w[5 + t1], w[5 + t2], sc.gamma);
-          R tt = dx_of<R>(p, d) / (Tr<R>::abs(w[1 + d]) + cf);
+          R tt = Tr<R>::div(dx_of<R>(p, d), Tr<R>::abs(w[1 + d]) + cf);
           m = rmin(m, tt);
         }
       }
@@ -288,7 +289,7 @@ __global__ void __launch_bounds__(kThreads) k_prim(const DPatch* __restrict__ P,
       const int b = (a + 1) % 3, cc = (a + 2) % 3;
       arr(scr, p, SC_EN + a)[x] = w[1 + cc] * w[5 + b] - w[1 + b] * w[5 + cc];
     }
-    if (!(w[0] > R(0)) || !(w[4] > R(0))) raise_status(status, -4);
+    if (!Tr<R>::pos(w[0]) || !Tr<R>::pos(w[4])) raise_status(status, -4);
   }
   if constexpr (Cfl) {
     for (int o = 16; o > 0; o >>= 1) {
@@ -341,7 +342,7 @@ template <typename R, int a> __device__ __forceinline__ R edge_avg_at(const DPat
   R e10 = En[x - sc_];
   R e01 = En[x - sb];
   R e11 = En[x];
-  return R(0.25) * (e00 + e10 + e01 + e11);
+  return Tr<R>::quarter(e00 + e10 + e01 + e11);
 }
 
 template <typename R, int a> __device__ __forceinline__ void edge_avg(const DPatch& p, const Cell& c, R* scr) {
@@ -362,39 +363,72 @@ template <typename R> struct RegSlopes {
   }
 };
 
-// Limited slopes of one cell parked in shared memory: six float4 rows of
-// kThreads entries (axis d: rows 2d and 2d + 1), each thread its own column.
+// 8-value sets of one cell parked in shared memory as rows of 16-byte vectors,
+// kThreads to a row, each thread its own column (set d: FP32 rows 2d and
+// 2d + 1, FP64 rows 4d to 4d + 3).
 // The stores and loads are volatile asm, so that the compiler neither
 // forwards the stored values in registers nor moves a load above its store;
-// the slopes then do not stay live across the Hancock increment, which is
-// what holds the FP32 predictor's registers down.
-__device__ __forceinline__ void sts4(uint32_t a, float x, float y, float z, float w) {
-  asm volatile("st.shared.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(a), "f"(x), "f"(y), "f"(z), "f"(w));
+// the values then do not stay live across the Hancock increment, which is
+// what holds the predictor's registers down.
+__device__ __forceinline__ void sts16(uint32_t a, const float* v) {
+  asm volatile("st.shared.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(a), "f"(v[0]), "f"(v[1]), "f"(v[2]), "f"(v[3]));
 }
-__device__ __forceinline__ float4 lds4(uint32_t a) {
-  float4 v;
-  asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "r"(a));
-  return v;
+__device__ __forceinline__ void lds16(uint32_t a, float* v) {
+  asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];"
+               : "=f"(v[0]), "=f"(v[1]), "=f"(v[2]), "=f"(v[3])
+               : "r"(a));
 }
-struct SmemSlopes {
+__device__ __forceinline__ void sts16(uint32_t a, const double* v) {
+  asm volatile("st.shared.v2.f64 [%0], {%1, %2};" ::"r"(a), "d"(v[0]), "d"(v[1]));
+}
+__device__ __forceinline__ void lds16(uint32_t a, double* v) {
+  asm volatile("ld.shared.v2.f64 {%0, %1}, [%2];" : "=d"(v[0]), "=d"(v[1]) : "r"(a));
+}
+template <typename R> struct SmemSets {
+  static constexpr int W = 16 / (int)sizeof(R);  // values per vector
   uint32_t base;  // shared address of row 0, this thread's column
-  __device__ __forceinline__ void put(int d, const float (&v)[8]) const {
-    sts4(base + (2 * d) * kThreads * 16, v[0], v[1], v[2], v[3]);
-    sts4(base + (2 * d + 1) * kThreads * 16, v[4], v[5], v[6], v[7]);
+  __device__ __forceinline__ uint32_t row(int d, int k) const {
+    return base + (uint32_t)(d * (8 / W) + k) * kThreads * 16;
   }
-  __device__ __forceinline__ void get(int d, float (&out)[8]) const {
-    const float4 a = lds4(base + (2 * d) * kThreads * 16), b = lds4(base + (2 * d + 1) * kThreads * 16);
-    out[0] = a.x; out[1] = a.y; out[2] = a.z; out[3] = a.w;
-    out[4] = b.x; out[5] = b.y; out[6] = b.z; out[7] = b.w;
+  __device__ __forceinline__ void put(int d, const R (&v)[8]) const {
+#pragma unroll
+    for (int k = 0; k < 8 / W; ++k) sts16(row(d, k), v + k * W);
+  }
+  __device__ __forceinline__ void put2(int d, int k, double v0, double v1) const {
+    const double v[2] = {v0, v1};
+    sts16(row(d, k), v);
+  }
+  __device__ __forceinline__ void get(int d, R (&out)[8]) const {
+#pragma unroll
+    for (int k = 0; k < 8 / W; ++k) lds16(row(d, k), out + k * W);
   }
 };
 
-// First positivity rule on the face values of rho and p along one axis:
-// true if a face value is not positive.
+// First positivity rule on the face values of rho or p along one axis: true
+// if a face value is not positive (h: half the slope).
+template <typename R> __device__ __forceinline__ bool face_rule1(R w, R h) {
+  return !Tr<R>::pos(w - h) || !Tr<R>::pos(w + h);
+}
 template <typename R> __device__ __forceinline__ bool face_rule1(const R (&w)[8], const R (&dw)[8]) {
-  const R rm = w[0] - R(0.5) * dw[0], rp = w[0] + R(0.5) * dw[0];
-  const R pm = w[4] - R(0.5) * dw[4], pp = w[4] + R(0.5) * dw[4];
-  return !(rm > R(0)) || !(rp > R(0)) || !(pm > R(0)) || !(pp > R(0));
+  return face_rule1(w[0], Tr<R>::half(dw[0])) || face_rule1(w[4], Tr<R>::half(dw[4]));
+}
+
+// The reference cell EMFs from U^{n+1/2} = U(w) + du, read by the upwinded EMF
+// average only, stored at element x.
+template <typename R>
+__device__ __forceinline__ void reference_emf(const DPatch& p, int64_t x, R* scr, const SolverConsts<R>& sc,
+                                              const R (&w)[8], const R (&du)[8]) {
+  R uc[8], uh[8];
+  prim2cons(w, sc.igm1, uc);
+#pragma unroll
+  for (int q = 0; q < 8; ++q) uh[q] = uc[q] + du[q];
+  R ir = Tr<R>::div(R(1), uh[0]);
+  R v[3] = {uh[1] * ir, uh[2] * ir, uh[3] * ir};
+#pragma unroll
+  for (int a = 0; a < 3; ++a) {
+    const int b = (a + 1) % 3, cc = (a + 2) % 3;
+    arr(scr, p, SC_ER + a)[x] = v[cc] * uh[5 + b] - v[b] * uh[5 + cc];
+  }
 }
 
 // The predictor of one cell from its primitives w and limited slopes (S),
@@ -438,7 +472,7 @@ __device__ __forceinline__ void predict_cell(const DPatch& p, int64_t x, R* scr,
 #pragma unroll
       for (int q = 0; q < 8; ++q) u[q] = u[q] + du[q];
       cons2prim(u, sc.gm1, pw);
-      if (!(pw[0] > R(0)) || !(pw[4] > R(0))) bad2 = true;
+      if (!Tr<R>::pos(pw[0]) || !Tr<R>::pos(pw[4])) bad2 = true;
       store_face_state(arr(scr, p, SC_WF + (d * 2 + sd) * 8), p.snelem, x, d, pw);
     }
   }
@@ -451,35 +485,41 @@ __device__ __forceinline__ void predict_cell(const DPatch& p, int64_t x, R* scr,
 #pragma unroll
     for (int q = 0; q < 8; ++q) duk[q] = R(0);
   }
-  // reference cell EMF from U^{n+1/2} (read only by the upwinded EMF average)
-  if (sc.emf == 1) return;
-  R uc[8], uh[8];
-  prim2cons(w, sc.igm1, uc);
-#pragma unroll
-  for (int q = 0; q < 8; ++q) uh[q] = uc[q] + duk[q];
-  R ir = R(1) / uh[0];
-  R v[3] = {uh[1] * ir, uh[2] * ir, uh[3] * ir};
-#pragma unroll
-  for (int a = 0; a < 3; ++a) {
-    const int b = (a + 1) % 3, cc = (a + 2) % 3;
-    arr(scr, p, SC_ER + a)[x] = v[cc] * uh[5 + b] - v[b] * uh[5 + cc];
-  }
+  if (sc.emf != 1) reference_emf(p, x, scr, sc, w, duk);
+}
+
+// Vector k (of 16 bytes) of the primitives of element x.
+__device__ __forceinline__ void load_wvec(const float* g, int64_t sn, int64_t x, int k, float (&v)[4]) {
+  const float4 a = reinterpret_cast<const float4*>(g + 4 * k * sn)[x];
+  v[0] = a.x; v[1] = a.y; v[2] = a.z; v[3] = a.w;
+}
+__device__ __forceinline__ void load_wvec(const double* g, int64_t sn, int64_t x, int k, double (&v)[2]) {
+  const double2 a = reinterpret_cast<const double2*>(g + 2 * k * sn)[x];
+  v[0] = a.x; v[1] = a.y;
 }
 
 // One thread per cell of UB+1; the stencil of W is read from the scratch
-// planes through the caches.  FP32 parks the slopes in shared memory
-// (SmemSlopes) and is held at 80 registers, three blocks per SM (measured on
-// GB300: 132 us against 136 us with the slopes in registers at 117 registers
-// and two blocks); FP64 keeps them in registers at one block per SM, its
-// time being set by the FP64 pipe.  The FP32 flux kernel is held at 64
-// registers (four blocks per SM): past that the compiler's choice drops a
-// block per SM and the kernel, bound by the latency of its loads, slows down.
+// planes through the caches, and what a thread needs again later is parked in
+// shared memory (SmemSets).
+//
+// FP32 parks the slopes and is held at 80 registers, three blocks per SM
+// (measured on GB300: 132 us against 136 us with the slopes in registers at
+// 117 registers and two blocks).
+//
+// FP64 is bound by the FP64 pipe, so it parks the conserved face
+// states: they are computed once, with the flux of their face, and the second
+// phase adds the Hancock increment to them.  The slopes are taken in a rolled
+// loop, whose 60-instruction divisions would overflow the instruction cache
+// unrolled, into the rows of the first face of their axis.  Measured on the
+// 128^3 blast (contracted, integer divisions): slopes in registers at one
+// block per SM 3.21 ms, slopes parked at two blocks 2.29 ms, face states
+// parked 1.97 ms, then 85% of the FP64 pipe; three blocks gain nothing more.
 template <typename R>
-__global__ void __launch_bounds__(kThreads, sizeof(R) == 4 ? MHD_PRED_MINB : 1) k_pred(const DPatch* __restrict__ P,
+__global__ void __launch_bounds__(kThreads, sizeof(R) == 4 ? MHD_PRED_MINB : 2) k_pred(const DPatch* __restrict__ P,
                                                    const BlockTask* __restrict__ T, R* scr,
                                                    SolverConsts<R> sc, const R* __restrict__ K) {
-  constexpr bool smem = sizeof(R) == 4;
-  __shared__ float4 sdw[smem ? 6 : 1][smem ? kThreads : 1];
+  using S = SmemSets<R>;
+  extern __shared__ __align__(16) unsigned char pred_smem[];
   const BlockTask t = T[blockIdx.x];
   const DPatch& p = P[t.patch];
   Cell c;
@@ -487,25 +527,87 @@ __global__ void __launch_bounds__(kThreads, sizeof(R) == 4 ? MHD_PRED_MINB : 1) 
   if (kM1<R> > 1 && (!in_ub(p, 0, c.i, -1, 1) || !in_ub(p, 1, c.j, -1, 1) || !in_ub(p, 2, c.k, -1, 1))) return;
   const StepDt<R> st(K, t.patch);
   const int64_t x = lin(p, c);
-  R w[8], dw[3][8];
   const R* Wg = arr(scr, p, SC_W);
+  const S ss{(uint32_t)__cvta_generic_to_shared(pred_smem) + threadIdx.x * 16};
+  R w[8];
   VecIO<R>::load8(Wg, p.snelem, x, w);
-  SmemSlopes ss{(uint32_t)__cvta_generic_to_shared(&sdw[0][smem ? threadIdx.x : 0])};
   bool bad = false;
+  if constexpr (sizeof(R) == 4) {
 #pragma unroll
-  for (int d = 0; d < 3; ++d) {
-    const int64_t sd = stride_of(p, d);
-    R wm[8], wp[8];
-    VecIO<R>::load8(Wg, p.snelem, x - sd, wm);
-    VecIO<R>::load8(Wg, p.snelem, x + sd, wp);
+    for (int d = 0; d < 3; ++d) {
+      const int64_t sd = stride_of(p, d);
+      R wm[8], wp[8], dw[8];
+      VecIO<R>::load8(Wg, p.snelem, x - sd, wm);
+      VecIO<R>::load8(Wg, p.snelem, x + sd, wp);
 #pragma unroll
-    for (int q = 0; q < 8; ++q) dw[d][q] = limiter(sc.limiter, w[q] - wm[q], wp[q] - w[q]);
-    if (face_rule1(w, dw[d])) bad = true;
-    if constexpr (smem) ss.put(d, dw[d]);
+      for (int q = 0; q < 8; ++q) dw[q] = limiter(sc.limiter, w[q] - wm[q], wp[q] - w[q]);
+      if (face_rule1(w, dw)) bad = true;
+      ss.put(d, dw);
+    }
+    predict_cell(p, x, scr, sc, st, w, ss, bad);
+  } else {
+    R du[8];
+#pragma unroll
+    for (int d = 0; d < 3; ++d) {
+      const int64_t sd = stride_of(p, d);
+#pragma unroll 1
+      for (int k = 0; k < 4; ++k) {  // two half slopes at a time
+        const R* g = Wg + 2 * k * p.snelem;
+        const double2 v = reinterpret_cast<const double2*>(g)[x], vm = reinterpret_cast<const double2*>(g)[x - sd],
+                      vp = reinterpret_cast<const double2*>(g)[x + sd];
+        const double hx = half_slope(sc.limiter, v.x - vm.x, vp.x - v.x);
+        const double hy = half_slope(sc.limiter, v.y - vm.y, vp.y - v.y);
+        ss.put2(2 * d, k, hx, hy);
+        if (k % 2 == 0 && face_rule1(v.x, hx)) bad = true;  // rho, p
+      }
+      R h[8], fw[8], u[8], fm[8], fp[8];
+      ss.get(2 * d, h);
+#pragma unroll
+      for (int q = 0; q < 8; ++q) fw[q] = w[q] - h[q];
+      cons_flux<kFastRecip>(d, fw, sc.igm1, u, fm);
+      ss.put(2 * d, u);
+#pragma unroll
+      for (int q = 0; q < 8; ++q) fw[q] = w[q] + h[q];
+      cons_flux<kFastRecip>(d, fw, sc.igm1, u, fp);
+      ss.put(2 * d + 1, u);
+#pragma unroll
+      for (int q = 0; q < 8; ++q) {  // the normal-B flux along an axis is zero
+        const R df = q == 5 + d ? R(0) : st.hdtdx[d] * (fp[q] - fm[q]);
+        du[q] = d == 0 ? -df : du[q] - df;
+      }
+    }
+    if (bad) {  // first positivity rule: zero slopes, hence no increment
+      R u[8];
+      prim2cons(w, sc.igm1, u);
+#pragma unroll 1
+      for (int f = 0; f < 6; ++f) ss.put(f, u);
+#pragma unroll
+      for (int q = 0; q < 8; ++q) du[q] = R(0);
+    }
+    bool bad2 = false;
+#pragma unroll 1
+    for (int f = 0; f < 6; ++f) {
+      R u[8], pw[8];
+      ss.get(f, u);
+#pragma unroll
+      for (int q = 0; q < 8; ++q) u[q] = u[q] + du[q];
+      cons2prim(u, sc.gm1, pw);
+      if (!Tr<R>::pos(pw[0]) || !Tr<R>::pos(pw[4])) bad2 = true;
+      store_face_state(arr(scr, p, SC_WF + f * 8), p.snelem, x, f >> 1, pw);
+    }
+    if (bad2) {  // second positivity rule: first order
+#pragma unroll 1
+      for (int f = 0; f < 6; ++f) store_face_state(arr(scr, p, SC_WF + f * 8), p.snelem, x, f >> 1, w);
+#pragma unroll
+      for (int q = 0; q < 8; ++q) du[q] = R(0);
+    }
+    if (sc.emf != 1) reference_emf(p, x, scr, sc, w, du);
   }
-  if constexpr (smem) predict_cell(p, x, scr, sc, st, w, ss, bad);
-  else predict_cell(p, x, scr, sc, st, w, RegSlopes<R>{dw}, bad);
 }
+
+// Dynamic shared memory of k_pred: FP32 the slopes of three axes, FP64 six
+// conserved face states.
+template <typename R> constexpr size_t kPredSmem = sizeof(R) * (sizeof(R) == 4 ? 24 : 48) * kThreads;
 
 // Tiled predictor: a block owns a TX x TY x TZ tile of UB+1 cells (its task's
 // `start` is the tile index within the patch), stages W on the tile grown by
@@ -605,7 +707,7 @@ __device__ __forceinline__ void flux_face(const DPatch& p, int patch, const Cell
   VecIO<R>::load7(arr(scr, p, SC_WF + (d * 2 + 0) * 8), p.snelem, x, vr);
   const R L[8] = {vl[0], vl[1], vl[2], vl[3], vl[4], R(0), vl[5], vl[6]};
   const R Rr[8] = {vr[0], vr[1], vr[2], vr[3], vr[4], R(0), vr[5], vr[6]};
-  hlld<R, kFastRecip>(L, Rr, bh, sc.gamma, sc.igm1, sc.eps_up, fr, &upw);
+  hlld<R, kFastRecip>(L, Rr, bh, sc.gamma, sc.igm1, sc.eps_up, sc.emf != 1, fr, &upw);
   rot_out(d, fr, f);
   f[5 + d] = upw;
   VecIO<R>::store8(arr(scr, p, SC_F + d * 8), p.snelem, x, f);
@@ -632,22 +734,22 @@ __global__ void __launch_bounds__(kThreads, sizeof(R) == 4 ? 4 : 2) k_flux(const
 template <typename R>
 __device__ __forceinline__ R edge_emf_value(R eb_lo, R eb_hi, R ec_lo, R ec_hi, R r00, R r10, R r01, R r11,
                                             R mb_lo, R mb_hi, R mc_lo, R mc_hi, int emf) {
-  R avg = R(0.25) * (eb_lo + eb_hi + ec_lo + ec_hi);
+  R avg = Tr<R>::quarter(eb_lo + eb_hi + ec_lo + ec_hi);
   if (emf == 1) return avg;
   R dc14, dc34, db14, db34;
-  if (mb_hi > R(0)) dc14 = r01 - ec_lo;
-  else if (mb_hi < R(0)) dc14 = r11 - ec_hi;
-  else dc14 = R(0.5) * ((r01 - ec_lo) + (r11 - ec_hi));
-  if (mb_lo > R(0)) dc34 = ec_lo - r00;
-  else if (mb_lo < R(0)) dc34 = ec_hi - r10;
-  else dc34 = R(0.5) * ((ec_lo - r00) + (ec_hi - r10));
-  if (mc_hi > R(0)) db14 = r10 - eb_lo;
-  else if (mc_hi < R(0)) db14 = r11 - eb_hi;
-  else db14 = R(0.5) * ((r10 - eb_lo) + (r11 - eb_hi));
-  if (mc_lo > R(0)) db34 = eb_lo - r00;
-  else if (mc_lo < R(0)) db34 = eb_hi - r01;
-  else db34 = R(0.5) * ((eb_lo - r00) + (eb_hi - r01));
-  return avg + R(0.25) * (dc34 - dc14 + db34 - db14);
+  if (Tr<R>::pos(mb_hi)) dc14 = r01 - ec_lo;
+  else if (Tr<R>::neg(mb_hi)) dc14 = r11 - ec_hi;
+  else dc14 = Tr<R>::half((r01 - ec_lo) + (r11 - ec_hi));
+  if (Tr<R>::pos(mb_lo)) dc34 = ec_lo - r00;
+  else if (Tr<R>::neg(mb_lo)) dc34 = ec_hi - r10;
+  else dc34 = Tr<R>::half((ec_lo - r00) + (ec_hi - r10));
+  if (Tr<R>::pos(mc_hi)) db14 = r10 - eb_lo;
+  else if (Tr<R>::neg(mc_hi)) db14 = r11 - eb_hi;
+  else db14 = Tr<R>::half((r10 - eb_lo) + (r11 - eb_hi));
+  if (Tr<R>::pos(mc_lo)) db34 = eb_lo - r00;
+  else if (Tr<R>::neg(mc_lo)) db34 = eb_hi - r01;
+  else db34 = Tr<R>::half((eb_lo - r00) + (eb_hi - r01));
+  return avg + Tr<R>::quarter(dc34 - dc14 + db34 - db14);
 }
 
 // EMF of the axis-a edge stored at element x: the face EMFs -F_b[B_c] of the
@@ -663,7 +765,7 @@ __device__ __forceinline__ R emf_at(const DPatch& p, int64_t x, const R* scr, in
   const R* Fc = arr(scr, p, SC_F + cc * 8);
   const R eb_lo = -*vgroup_at(Fb, sn, x - scc, 5 + cc), eb_hi = -*vgroup_at(Fb, sn, x, 5 + cc);
   const R ec_lo = *vgroup_at(Fc, sn, x - sb, 5 + b), ec_hi = *vgroup_at(Fc, sn, x, 5 + b);
-  if (emf == 1) return R(0.25) * (eb_lo + eb_hi + ec_lo + ec_hi);
+  if (emf == 1) return Tr<R>::quarter(eb_lo + eb_hi + ec_lo + ec_hi);
   const R* Er = arr(scr, p, SC_ER + a);
   return edge_emf_value(eb_lo, eb_hi, ec_lo, ec_hi, Er[x - sb - scc], Er[x - scc], Er[x - sb], Er[x],
                         *vgroup_at(Fb, sn, x - scc, 5 + b), *vgroup_at(Fb, sn, x, 5 + b),
@@ -862,9 +964,9 @@ __device__ __forceinline__ bool floor_cell(const DPatch& p, int64_t x, const Sol
   R u[8], w[8];
 #pragma unroll
   for (int q = 0; q < 5; ++q) u[q] = ((const R*)p.U[q])[x];
-  u[5] = R(0.5) * (((const R*)p.B[0])[x] + ((const R*)p.B[0])[x + 1]);
-  u[6] = R(0.5) * (((const R*)p.B[1])[x] + ((const R*)p.B[1])[x + p.s1]);
-  u[7] = R(0.5) * (((const R*)p.B[2])[x] + ((const R*)p.B[2])[x + p.s2]);
+  u[5] = Tr<R>::half(((const R*)p.B[0])[x] + ((const R*)p.B[0])[x + 1]);
+  u[6] = Tr<R>::half(((const R*)p.B[1])[x] + ((const R*)p.B[1])[x + p.s1]);
+  u[7] = Tr<R>::half(((const R*)p.B[2])[x] + ((const R*)p.B[2])[x + p.s2]);
   cons2prim(u, sc.gm1, w);
   if (sc.rho_floor > R(0) && !(w[0] >= sc.rho_floor)) {
     const R ke = R(0.5) * (u[1] * u[1] + u[2] * u[2] + u[3] * u[3]) / sc.rho_floor;
@@ -897,6 +999,19 @@ __global__ void __launch_bounds__(kThreads) k_floor(const DPatch* __restrict__ P
 
 #include "pf.cuh"
 
+// Lets kernel f use smem bytes of dynamic shared memory on the current device
+// (`configured`: the kernel's own flags, one per device).
+template <typename F> cudaError_t allow_smem(F f, size_t smem, bool (&configured)[64]) {
+  int dev = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e != cudaSuccess) return e;
+  if (dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
+  if (configured[dev]) return cudaSuccess;
+  e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  if (e == cudaSuccess) configured[dev] = true;
+  return e;
+}
+
 // Enqueues the step constants, the fused pass of compiled shape TX x TY and
 // the staged EMF / update / floor kernels.
 template <typename R, int TX, int TY, int MINB>
@@ -905,15 +1020,8 @@ cudaError_t launch_pf_shape(const AdvanceArgs& a, R* scr, R* K, const SolverCons
   if (a.npf == 0) return cudaSuccess;
   const size_t smem = sizeof(R) * L::TOTAL;
   static bool configured[64] = {};
-  int dev = 0;
-  cudaError_t e = cudaGetDevice(&dev);
+  const cudaError_t e = allow_smem(k_pf<R, TX, TY, MINB>, smem, configured);
   if (e != cudaSuccess) return e;
-  if (dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
-  if (!configured[dev]) {
-    e = cudaFuncSetAttribute(k_pf<R, TX, TY, MINB>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-    configured[dev] = true;
-  }
   const KernelTimer* tm = a.timer;
   MHD_TIMED(tm, K_PF, s,
             (k_stepc<R><<<(a.npatches + 127) / 128, 128, 0, s>>>(a.patches, a.npatches, a.d_dt, K),
@@ -976,7 +1084,12 @@ cudaError_t launch_advance(const AdvanceArgs& a, R* scr, R* K, const SolverConst
   if (npblocks > 0)
     MHD_TIMED(tm, K_PRED, s, (k_pred_tiled<R><<<npblocks, kThreads, 0, s>>>(d_patches, d_ptasks, scr, sc, K)));
   else
-    MHD_TIMED(tm, K_PRED, s, (k_pred<R><<<g1b, kThreads, 0, s>>>(d_patches, d_tasks1, scr, sc, K)));
+    {
+    static bool configured[64] = {};
+    const cudaError_t e = allow_smem(k_pred<R>, kPredSmem<R>, configured);
+    if (e != cudaSuccess) return e;
+    MHD_TIMED(tm, K_PRED, s, (k_pred<R><<<g1b, kThreads, kPredSmem<R>, s>>>(d_patches, d_tasks1, scr, sc, K)));
+  }
   constexpr bool inl = kInlineEdges<R>;
   if (!inl) MHD_TIMED(tm, K_EDGE, s, (k_edge<R><<<g1, kThreads, 0, s>>>(d_patches, d_tasks, scr)));
   MHD_TIMED(tm, K_FLUX, s, (k_flux<R><<<g1b, kThreads, 0, s>>>(d_patches, d_tasks1, scr, sc, K)));

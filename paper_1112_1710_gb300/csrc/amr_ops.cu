@@ -53,11 +53,11 @@ template <typename R> __device__ __forceinline__ R minmod(R a, R b) { return lim
 template <typename R> __device__ __forceinline__ R thermal(const DPatch& p, int64_t x) {
   const R rho = ((const R*)p.U[0])[x];
   const R mx = ((const R*)p.U[1])[x], my = ((const R*)p.U[2])[x], mz = ((const R*)p.U[3])[x];
-  R ke = R(0.5) * (mx * mx + my * my + mz * mz) / rho;
-  R bx = R(0.5) * (((const R*)p.B[0])[x] + ((const R*)p.B[0])[x + 1]);
-  R by = R(0.5) * (((const R*)p.B[1])[x] + ((const R*)p.B[1])[x + p.s1]);
-  R bz = R(0.5) * (((const R*)p.B[2])[x] + ((const R*)p.B[2])[x + p.s2]);
-  R me = R(0.5) * (bx * bx + by * by + bz * bz);
+  R ke = Tr<R>::div(Tr<R>::half(mx * mx + my * my + mz * mz), rho);
+  R bx = Tr<R>::half(((const R*)p.B[0])[x] + ((const R*)p.B[0])[x + 1]);
+  R by = Tr<R>::half(((const R*)p.B[1])[x] + ((const R*)p.B[1])[x + p.s1]);
+  R bz = Tr<R>::half(((const R*)p.B[2])[x] + ((const R*)p.B[2])[x + p.s2]);
+  R me = Tr<R>::half(bx * bx + by * by + bz * bz);
   return ((const R*)p.U[4])[x] - ke - me;
 }
 
@@ -271,7 +271,7 @@ __global__ void __launch_bounds__(kThreads, sizeof(R) == 4 ? MHD_PROLONG_MINB : 
     for (int d = 0; d < 3; ++d) {
       R a = uc[q] - Uq[c - sof(pc, d)];
       R b = Uq[c + sof(pc, d)] - uc[q];
-      h[q][d] = R(0.25) * minmod(a, b);
+      h[q][d] = Tr<R>::quarter(minmod(a, b));
     }
   }
   const R ec = thermal<R>(pc, c);
@@ -279,7 +279,7 @@ __global__ void __launch_bounds__(kThreads, sizeof(R) == 4 ? MHD_PROLONG_MINB : 
   for (int d = 0; d < 3; ++d) {
     R a = ec - thermal<R>(pc, c - sof(pc, d));
     R b = thermal<R>(pc, c + sof(pc, d)) - ec;
-    he[d] = R(0.25) * minmod(a, b);
+    he[d] = Tr<R>::quarter(minmod(a, b));
   }
   R m[3][2], qs[3][2][3];
 #pragma unroll
@@ -297,7 +297,7 @@ __global__ void __launch_bounds__(kThreads, sizeof(R) == 4 ? MHD_PROLONG_MINB : 
         }
         R lo = m[a][sd] - Ba[f - sof(pc, tt)];
         R hi = Ba[f + sof(pc, tt)] - m[a][sd];
-        qs[a][sd][tt] = R(0.25) * minmod(lo, hi);
+        qs[a][sd][tt] = Tr<R>::quarter(minmod(lo, hi));
       }
     }
   }
@@ -366,7 +366,7 @@ __global__ void __launch_bounds__(kThreads, sizeof(R) == 4 ? MHD_PROLONG_MINB : 
         e = e + (fa ? he[0] : -he[0]);
         e = e + (fb ? he[1] : -he[1]);
         e = e + (fc ? he[2] : -he[2]);
-        const R kef = R(0.5) * (uf[fa][1] * uf[fa][1] + uf[fa][2] * uf[fa][2] + uf[fa][3] * uf[fa][3]) / uf[fa][0];
+        const R kef = Tr<R>::div(Tr<R>::half(uf[fa][1] * uf[fa][1] + uf[fa][2] * uf[fa][2] + uf[fa][3] * uf[fa][3]), uf[fa][0]);
         const R mef = R(0.5) * (bc[0] * bc[0] + bc[1] * bc[1] + bc[2] * bc[2]);
         en[fa] = e + kef + mef;
       }

@@ -63,9 +63,9 @@ __device__ __forceinline__ void fused_prim(const DPatch& p, R* sm, int X0, int Y
     R u[8];
 #pragma unroll
     for (int q = 0; q < 5; ++q) u[q] = ((const R*)p.U[q])[x];
-    u[5] = R(0.5) * (((const R*)p.B[0])[x] + ((const R*)p.B[0])[x + 1]);
-    u[6] = R(0.5) * (((const R*)p.B[1])[x] + ((const R*)p.B[1])[x + p.s1]);
-    u[7] = R(0.5) * (((const R*)p.B[2])[x] + ((const R*)p.B[2])[x + p.s2]);
+    u[5] = Tr<R>::half(((const R*)p.B[0])[x] + ((const R*)p.B[0])[x + 1]);
+    u[6] = Tr<R>::half(((const R*)p.B[1])[x] + ((const R*)p.B[1])[x + p.s1]);
+    u[7] = Tr<R>::half(((const R*)p.B[2])[x] + ((const R*)p.B[2])[x + p.s2]);
     R w[8];
     cons2prim(u, sc.gm1, w);
     if (sc.rho_floor > R(0) && !(w[0] >= sc.rho_floor)) w[0] = sc.rho_floor;
@@ -180,7 +180,7 @@ __device__ __forceinline__ void fused_pred(R* sm, int TX, int TY, int z, const S
     prim2cons(w, sc.igm1, uc);
 #pragma unroll
     for (int q = 0; q < 8; ++q) uh[q] = uc[q] + du[q];
-    R ir = R(1) / uh[0];
+    R ir = Tr<R>::div(R(1), uh[0]);
     R v[3] = {uh[1] * ir, uh[2] * ir, uh[3] * ir};
 #pragma unroll
     for (int a = 0; a < 3; ++a) {
@@ -212,14 +212,14 @@ __device__ __forceinline__ void fused_edges(R* sm, int TX, int TY, int ze, bool 
         R e10 = Em[0 * L::G2 + s];
         R e01 = E0[0 * L::G2 + s - L::P2];
         R e11 = E0[0 * L::G2 + s];
-        EXY[0 * L::GE + se] = R(0.25) * (e00 + e10 + e01 + e11);
+        EXY[0 * L::GE + se] = Tr<R>::quarter(e00 + e10 + e01 + e11);
       }
       {  // y-edge: cells (i-1, k-1), (i-1, k), (i, k-1), (i, k)
         R e00 = Em[1 * L::G2 + s - 1];
         R e10 = E0[1 * L::G2 + s - 1];
         R e01 = Em[1 * L::G2 + s];
         R e11 = E0[1 * L::G2 + s];
-        EXY[1 * L::GE + se] = R(0.25) * (e00 + e10 + e01 + e11);
+        EXY[1 * L::GE + se] = Tr<R>::quarter(e00 + e10 + e01 + e11);
       }
     }
     if (do_z) {  // z-edge: cells (i-1, j-1), (i, j-1), (i-1, j), (i, j)
@@ -227,7 +227,7 @@ __device__ __forceinline__ void fused_edges(R* sm, int TX, int TY, int ze, bool 
       R e10 = Ez[s - L::P2];
       R e01 = Ez[s - 1];
       R e11 = Ez[s];
-      EZ[se] = R(0.25) * (e00 + e10 + e01 + e11);
+      EZ[se] = Tr<R>::quarter(e00 + e10 + e01 + e11);
     }
   }
 }
@@ -239,7 +239,7 @@ __device__ __forceinline__ void face_flux(const R* wl, const R* wr, R bh, const 
   R L[8], Rr[8], fr[8], upw;
   rot_in(d, wl, L);
   rot_in(d, wr, Rr);
-  hlld<R, kFastRecip>(L, Rr, bh, sc.gamma, sc.igm1, sc.eps_up, fr, &upw);
+  hlld<R, kFastRecip>(L, Rr, bh, sc.gamma, sc.igm1, sc.eps_up, sc.emf != 1, fr, &upw);
   rot_out(d, fr, f);
   f[5 + d] = upw;
 }

@@ -46,15 +46,15 @@ __global__ void __launch_bounds__(kThreads) k_cfl(const DPatch* __restrict__ P,
     R u[8], w[8];
 #pragma unroll
     for (int q = 0; q < 5; ++q) u[q] = ((const R*)p.U[q])[x];
-    u[5] = R(0.5) * (((const R*)p.B[0])[x] + ((const R*)p.B[0])[x + 1]);
-    u[6] = R(0.5) * (((const R*)p.B[1])[x] + ((const R*)p.B[1])[x + p.s1]);
-    u[7] = R(0.5) * (((const R*)p.B[2])[x] + ((const R*)p.B[2])[x + p.s2]);
+    u[5] = Tr<R>::half(((const R*)p.B[0])[x] + ((const R*)p.B[0])[x + 1]);
+    u[6] = Tr<R>::half(((const R*)p.B[1])[x] + ((const R*)p.B[1])[x + p.s1]);
+    u[7] = Tr<R>::half(((const R*)p.B[2])[x] + ((const R*)p.B[2])[x + p.s2]);
     cons2prim(u, gm1, w);
 #pragma unroll
     for (int d = 0; d < 3; ++d) {
       const int t1 = (d + 1) % 3, t2 = (d + 2) % 3;
       R cf = fast_speed(w[0], w[4], w[5 + d], w[5 + t1], w[5 + t2], gamma);
-      R tt = dx_of<R>(p, d) / (Tr<R>::abs(w[1 + d]) + cf);
+      R tt = Tr<R>::div(dx_of<R>(p, d), Tr<R>::abs(w[1 + d]) + cf);
       m = rmin(m, tt);
     }
     if (!(w[0] > R(0)) || !(w[4] > R(0))) raise_status(status, -4);

@@ -164,7 +164,7 @@ __device__ __forceinline__ R pf_edge(const R* __restrict__ sm, int s, int z) {
     e01 = E0[s - so[b]];
     e11 = E0[s];
   }
-  return R(0.25) * (e00 + e10 + e01 + e11);
+  return Tr<R>::quarter(e00 + e10 + e01 + e11);
 }
 
 // The flux of the axis-d lower face of tile cell c (position fx, fy on plane
@@ -212,7 +212,7 @@ __device__ __forceinline__ void pf_face(const R* __restrict__ sm, const DPatch& 
   Lf[5] = R(0);
   Rf[5] = R(0);
   R fr[8], f[8], upw;
-  hlld<R, kFastRecip>(Lf, Rf, bh, sc.gamma, sc.igm1, sc.eps_up, fr, &upw);
+  hlld<R, kFastRecip>(Lf, Rf, bh, sc.gamma, sc.igm1, sc.eps_up, sc.emf != 1, fr, &upw);
   rot_out(d, fr, f);
   f[5 + d] = upw;
   VecIO<R>::store8(arr(scr, p, SC_F + d * 8), p.snelem, x, f);
@@ -268,9 +268,9 @@ __global__ void __launch_bounds__(PfLayout<TX, TY>::NT, MINB)
       R u[8];
 #pragma unroll
       for (int q = 0; q < 5; ++q) u[q] = ((const R*)p.U[q])[x];
-      u[5] = R(0.5) * (((const R*)p.B[0])[x] + ((const R*)p.B[0])[x + 1]);
-      u[6] = R(0.5) * (((const R*)p.B[1])[x] + ((const R*)p.B[1])[x + s1]);
-      u[7] = R(0.5) * (((const R*)p.B[2])[x] + ((const R*)p.B[2])[x + s2]);
+      u[5] = Tr<R>::half(((const R*)p.B[0])[x] + ((const R*)p.B[0])[x + 1]);
+      u[6] = Tr<R>::half(((const R*)p.B[1])[x] + ((const R*)p.B[1])[x + s1]);
+      u[7] = Tr<R>::half(((const R*)p.B[2])[x] + ((const R*)p.B[2])[x + s2]);
       R w[8];
       cons2prim(u, sc.gm1, w);
       if (sc.rho_floor > R(0) && !(w[0] >= sc.rho_floor)) w[0] = sc.rho_floor;
@@ -313,7 +313,7 @@ __global__ void __launch_bounds__(PfLayout<TX, TY>::NT, MINB)
           prim2cons(w, sc.igm1, uc);
 #pragma unroll
           for (int q = 0; q < 8; ++q) uh[q] = uc[q] + duk[q];
-          R ir = R(1) / uh[0];
+          R ir = Tr<R>::div(R(1), uh[0]);
           R v[3] = {uh[1] * ir, uh[2] * ir, uh[3] * ir};
 #pragma unroll
           for (int a = 0; a < 3; ++a) {

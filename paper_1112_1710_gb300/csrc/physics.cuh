@@ -14,8 +14,14 @@
 
 #include <cstdint>
 
+#include "int64div.cuh"
+
 namespace mhd {
 
+// Arithmetic of each type.  FP64 divisions, square roots, sign tests and
+// scalings by powers of two run on the integer pipe (int64div.cuh): the FP64
+// pipe bounds every FP64 stage and the integer pipe idles.  The results have
+// the bits of the FP64 instructions.  div2: (a + a) / b.  flip: -x where c.
 // degen: relative threshold of the HLLD single-star degeneracy test.  It must
 // sit well above the rounding of rho (S - u)(S - S_M) - Bn^2 in the arithmetic
 // type: 1e-12 in FP64 (about 4500 ulp), 1e-5 in FP32 (about 80 ulp); an FP32
@@ -24,16 +30,45 @@ namespace mhd {
 template <typename R> struct Tr;
 template <> struct Tr<double> {
   __device__ static __forceinline__ double abs(double x) { return fabs(x); }
-  __device__ static __forceinline__ double sqrt_(double x) { return sqrt(x); }
-  __device__ static __forceinline__ double rsqrt_(double x) { return rsqrt(x); }
+  __device__ static __forceinline__ double sqrt_(double x) { return i64::sqrt_rn(x); }
+  __device__ static __forceinline__ double div(double a, double b) { return i64::div(a, b); }
+  __device__ static __forceinline__ double div2(double a, double b) { return i64::div_scaled<1>(a, b); }
+  __device__ static __forceinline__ double half(double x) { return i64::scale<-1>(x); }
+  __device__ static __forceinline__ double quarter(double x) { return i64::scale<-2>(x); }
+  __device__ static __forceinline__ double times2(double x) { return i64::scale<1>(x); }
+  __device__ static __forceinline__ double times4(double x) { return i64::scale<2>(x); }
+  __device__ static __forceinline__ bool pos(double x) { return i64::pos(x); }
+  __device__ static __forceinline__ bool neg(double x) { return i64::neg(x); }
+  __device__ static __forceinline__ bool ge0(double x) { return i64::ge0(x); }
+  __device__ static __forceinline__ bool abs_gt(double x, double t) { return i64::abs_gt(x, t); }
+  __device__ static __forceinline__ bool less_mag(double a, double b) { return i64::less_mag(a, b); }
   __device__ static __forceinline__ double degen() { return 1e-12; }
+  // |den| <= degen max(a1 a2, b); the exponents settle it almost always
+  __device__ static __forceinline__ bool degenerate(double den, double a1, double a2, double b) {
+    return !i64::clearly_above(den, a1, a2, b) && fabs(den) <= degen() * ((a1 * a2 > b) ? a1 * a2 : b);
+  }
 };
 template <> struct Tr<float> {
   __device__ static __forceinline__ float abs(float x) { return fabsf(x); }
   __device__ static __forceinline__ float sqrt_(float x) { return sqrtf(x); }
   __device__ static __forceinline__ float rsqrt_(float x) { return rsqrtf(x); }
+  __device__ static __forceinline__ float div(float a, float b) { return a / b; }
+  __device__ static __forceinline__ float div2(float a, float b) { return (a + a) / b; }
+  __device__ static __forceinline__ float half(float x) { return 0.5f * x; }
+  __device__ static __forceinline__ float quarter(float x) { return 0.25f * x; }
+  __device__ static __forceinline__ float times2(float x) { return 2.0f * x; }
+  __device__ static __forceinline__ float times4(float x) { return 4.0f * x; }
+  __device__ static __forceinline__ bool pos(float x) { return x > 0.0f; }
+  __device__ static __forceinline__ bool neg(float x) { return x < 0.0f; }
+  __device__ static __forceinline__ bool ge0(float x) { return x >= 0.0f; }
+  __device__ static __forceinline__ bool abs_gt(float x, float t) { return fabsf(x) > t; }
+  __device__ static __forceinline__ bool less_mag(float a, float b) { return fabsf(a) < fabsf(b); }
   __device__ static __forceinline__ float degen() { return 1e-5f; }
+  __device__ static __forceinline__ bool degenerate(float den, float a1, float a2, float b) {
+    return fabsf(den) <= degen() * fmaxf(a1 * a2, b);
+  }
 };
+template <typename R> __device__ __forceinline__ R flip(R x, bool c) { return c ? -x : x; }
 
 template <typename R> __device__ __forceinline__ R rmin(R a, R b) { return (a < b) ? a : b; }
 template <typename R> __device__ __forceinline__ R rmax(R a, R b) { return (a > b) ? a : b; }
@@ -42,23 +77,31 @@ template <typename R> __device__ __forceinline__ R rmax(R a, R b) { return (a > 
 // a*b <= 0 gives zero.
 template <typename R> __device__ __forceinline__ R limiter(int lim, R a, R b) {
   R ab = a * b;
-  if (!(ab > R(0))) return R(0);
-  if (lim == 1) return (Tr<R>::abs(a) < Tr<R>::abs(b)) ? a : b;
+  if (!Tr<R>::pos(ab)) return R(0);
+  if (lim == 1) return Tr<R>::less_mag(a, b) ? a : b;
   if (lim == 2) {
-    R s = (a > R(0)) ? R(1) : R(-1);
-    R m = rmin(rmin(R(2) * Tr<R>::abs(a), R(2) * Tr<R>::abs(b)), R(0.5) * Tr<R>::abs(a + b));
-    return s * m;
+    const R ma = Tr<R>::abs(a), mb = Tr<R>::abs(b);
+    const R t = Tr<R>::times2(Tr<R>::less_mag(a, b) ? ma : mb), h = Tr<R>::half(Tr<R>::abs(a + b));
+    return flip(Tr<R>::less_mag(t, h) ? t : h, Tr<R>::neg(a));
   }
-  return (ab + ab) / (a + b);
+  return Tr<R>::div2(ab, a + b);
+}
+
+// Half the limited slope (what the face values add and subtract): the van
+// Leer form is one quotient, a b / (a + b).
+template <typename R> __device__ __forceinline__ R half_slope(int lim, R a, R b) {
+  if (lim != 0) return Tr<R>::half(limiter(lim, a, b));
+  const R ab = a * b;
+  return Tr<R>::pos(ab) ? Tr<R>::div(ab, a + b) : R(0);
 }
 
 // conserved (rho, M, E, Bc) -> primitive (rho, v, p, Bc)
 template <typename R> __device__ __forceinline__ void cons2prim(const R* u, R gm1, R* w) {
   R rho = u[0];
-  R ir = R(1) / rho;
+  R ir = Tr<R>::div(R(1), rho);
   R vx = u[1] * ir, vy = u[2] * ir, vz = u[3] * ir;
-  R ke = R(0.5) * rho * (vx * vx + vy * vy + vz * vz);
-  R me = R(0.5) * (u[5] * u[5] + u[6] * u[6] + u[7] * u[7]);
+  R ke = Tr<R>::half(rho) * (vx * vx + vy * vy + vz * vz);
+  R me = Tr<R>::half(u[5] * u[5] + u[6] * u[6] + u[7] * u[7]);
   w[0] = rho; w[1] = vx; w[2] = vy; w[3] = vz;
   w[4] = gm1 * (u[4] - ke - me);
   w[5] = u[5]; w[6] = u[6]; w[7] = u[7];
@@ -66,8 +109,8 @@ template <typename R> __device__ __forceinline__ void cons2prim(const R* u, R gm
 
 template <typename R> __device__ __forceinline__ void prim2cons(const R* w, R igm1, R* u) {
   R rho = w[0];
-  R ke = R(0.5) * rho * (w[1] * w[1] + w[2] * w[2] + w[3] * w[3]);
-  R me = R(0.5) * (w[5] * w[5] + w[6] * w[6] + w[7] * w[7]);
+  R ke = Tr<R>::half(rho) * (w[1] * w[1] + w[2] * w[2] + w[3] * w[3]);
+  R me = Tr<R>::half(w[5] * w[5] + w[6] * w[6] + w[7] * w[7]);
   u[0] = rho;
   u[1] = rho * w[1]; u[2] = rho * w[2]; u[3] = rho * w[3];
   u[4] = w[4] * igm1 + ke + me;
@@ -77,14 +120,14 @@ template <typename R> __device__ __forceinline__ void prim2cons(const R* w, R ig
 // Fast magnetosonic speed: c_f^2 = ((a^2+b^2) + sqrt((a^2+b^2)^2 - 4 a^2 b_n^2))/2.
 template <typename R>
 __device__ __forceinline__ R fast_speed(R rho, R p, R bn, R bt1, R bt2, R gamma) {
-  R ir = R(1) / rho;
+  R ir = Tr<R>::div(R(1), rho);
   R a2 = gamma * p * ir;
   R b2 = (bn * bn + bt1 * bt1 + bt2 * bt2) * ir;
   R bn2 = bn * bn * ir;
   R s = a2 + b2;
-  R d = s * s - R(4) * a2 * bn2;
-  if (d < R(0)) d = R(0);
-  return Tr<R>::sqrt_(R(0.5) * (s + Tr<R>::sqrt_(d)));
+  R d = s * s - Tr<R>::times4(a2) * bn2;
+  if (Tr<R>::neg(d)) d = R(0);
+  return Tr<R>::sqrt_(Tr<R>::half(s + Tr<R>::sqrt_(d)));
 }
 
 // Ideal-MHD flux along the normal of a rotated primitive state
@@ -93,9 +136,9 @@ __device__ __forceinline__ R fast_speed(R rho, R p, R bn, R bt1, R bt2, R gamma)
 template <typename R> __device__ __forceinline__ void flux_rot(const R* r, R bn, R igm1, R* f) {
   R rho = r[0], vn = r[1], vt1 = r[2], vt2 = r[3], p = r[4];
   R bt1 = r[6], bt2 = r[7];
-  R pm = R(0.5) * (bn * bn + bt1 * bt1 + bt2 * bt2);
+  R pm = Tr<R>::half(bn * bn + bt1 * bt1 + bt2 * bt2);
   R pt = p + pm;
-  R ke = R(0.5) * rho * (vn * vn + vt1 * vt1 + vt2 * vt2);
+  R ke = Tr<R>::half(rho) * (vn * vn + vt1 * vt1 + vt2 * vt2);
   R e = p * igm1 + ke + pm;
   R vb = vn * bn + vt1 * bt1 + vt2 * bt2;
   R mn_ = rho * vn;
@@ -129,36 +172,51 @@ template <typename R> __device__ __forceinline__ void flux_xyz(int d, const R* w
   rot_out(d, fr, f);
 }
 
+// The conserved state u of an xyz primitive state and its physical flux f
+// along axis d.  FR: the flux from the conserved values (momenta, energy and
+// magnetic pressure computed once for both); else the expressions of
+// prim2cons and flux_xyz, whose sums run in different orders.
+template <bool FR, typename R> __device__ __forceinline__ void cons_flux(int d, const R* w, R igm1, R* u, R* f) {
+  if constexpr (FR) {
+    const R mx = w[0] * w[1], my = w[0] * w[2], mz = w[0] * w[3];
+    const R me = Tr<R>::half(w[5] * w[5] + w[6] * w[6] + w[7] * w[7]);
+    u[0] = w[0];
+    u[1] = mx; u[2] = my; u[3] = mz;
+    u[4] = w[4] * igm1 + Tr<R>::half(mx * w[1] + my * w[2] + mz * w[3]) + me;
+    u[5] = w[5]; u[6] = w[6]; u[7] = w[7];
+    const R pt = w[4] + me, vn = w[1 + d], bn = w[5 + d], mn = u[1 + d];
+    const R vb = w[1] * w[5] + w[2] * w[6] + w[3] * w[7];
+    f[0] = mn;
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+      f[1 + c] = mn * w[1 + c] - bn * w[5 + c];
+      f[5 + c] = c == d ? R(0) : w[5 + c] * vn - bn * w[1 + c];
+    }
+    f[1 + d] = f[1 + d] + pt;
+    f[4] = (u[4] + pt) * vn - bn * vb;
+  } else {
+    prim2cons(w, igm1, u);
+    flux_xyz(d, w, igm1, f);
+  }
+}
+
 // a / b, or a * ib with ib = 1 / b computed once for several quotients (the
 // reciprocal form of the FP32 and the contracted FP64 builds; the parity
 // build divides, as the oracle does)
 template <bool FR, typename R> __device__ __forceinline__ R qdiv(R a, R b, R ib) {
   if constexpr (FR) return a * ib;
-  else return a / b;
+  else return Tr<R>::div(a, b);
 }
 template <bool FR, typename R> __device__ __forceinline__ R recip(R b) {
-  if constexpr (FR) return R(1) / b;
+  if constexpr (FR) return Tr<R>::div(R(1), b);
   else return R(0);
 }
 
-// HLLD flux (Miyoshi & Kusano 2005) between rotated primitive states L (lower
-// side) and R_ (upper side) with interface normal field bn.  Wave speeds
-// S_L = min(u_L,u_R) - max(cf), S_R = max(u_L,u_R) + max(cf); S_M, p_T* from
-// MK05 eqs. (38), (41); star states eqs. (43)-(48) with a degenerate branch
-// (|rho(S-u)(S-S_M) - Bn^2| <= degen max(rho(S-u)^2, Bn^2), degen 1e-12 in
-// FP64 and 1e-5 in FP32, keeps the outer
-// transverse v, B); Alfven speeds S* = S_M -/+ |Bn|/sqrt(rho*); double-star
-// states eqs. (59)-(63); left-closed region selection.  f gets the rotated
-// flux; *upw the upwind side of the contact (+1, -1, or 0 when
-// |S_M| <= eps_up (S_R - S_L)).  FR: quotients with a common denominator
-// multiply by its reciprocal, and |Bn|/sqrt(rho*) uses a reciprocal square
-// root (8 divisions per face instead of 18), and the single-star field factor
-// is written as 1 + rho (S - u)(S_M - u)/den, which is exactly 1 where
-// S_M = u (a plain reciprocal would turn x/x into x (1/x), off by an ulp,
-// and give a 2D problem a z-field of rounding noise).
-template <typename R, bool FR = false>
-__device__ __forceinline__ void hlld(const R* L, const R* Rr, R bn, R gamma, R igm1, R eps_up,
-                                     R* f, R* upw) {
+// FP32 HLLD (hlld64's formulas and reciprocal form): both sides of the fan in
+// full, every region's flux from F* = F + S (U* - U).
+template <typename R>
+__device__ __forceinline__ void hlld32(const R* L, const R* Rr, R bn, R gamma, R igm1, R eps_up,
+                                       R* f, R* upw) {
   R rl = L[0], ul = L[1], vl = L[2], wl_ = L[3], pl = L[4], byl = L[6], bzl = L[7];
   R rr = Rr[0], ur = Rr[1], vr = Rr[2], wr_ = Rr[3], pr = Rr[4], byr = Rr[6], bzr = Rr[7];
 
@@ -188,32 +246,25 @@ __device__ __forceinline__ void hlld(const R* L, const R* Rr, R bn, R gamma, R i
   R sdl = sl - ul, sdr = sr - ur;
   R rsl = sdl * rl, rsr = sdr * rr;
   R dd = rsr - rsl;
-  const R idd = recip<FR>(dd);
-  R sm = qdiv<FR>((rsr * ur - rsl * ul) - (ptr - ptl), dd, idd);
-  R pts = qdiv<FR>((rsr * ptl - rsl * ptr) + rsl * rsr * (ur - ul), dd, idd);
+  const R idd = R(1) / dd;
+  R sm = ((rsr * ur - rsl * ul) - (ptr - ptl)) * idd;
+  R pts = ((rsr * ptl - rsl * ptr) + rsl * rsr * (ur - ul)) * idd;
   R tie = eps_up * (sr - sl);
   *upw = (sm > tie) ? R(1) : ((sm < -tie) ? R(-1) : R(0));
 
   R sml = sl - sm, smr = sr - sm;
-  const R isml = recip<FR>(sml), ismr = recip<FR>(smr);
-  R rls = qdiv<FR>(rsl, sml, isml), rrs = qdiv<FR>(rsr, smr, ismr);
+  const R isml = R(1) / sml, ismr = R(1) / smr;
+  R rls = rsl * isml, rrs = rsr * ismr;
   R bn2 = bn * bn;
   R vls, wls, byls, bzls;
   R denl = rsl * sml - bn2;
   if (Tr<R>::abs(denl) <= Tr<R>::degen() * rmax(rsl * sdl, bn2)) {
     vls = vl; wls = wl_; byls = byl; bzls = bzl;
   } else {
-    R fv, fb;
-    if constexpr (FR) {
-      // numerator of fb = den + rho (S - u)(S_M - u): fb = 1 + rho (S - u) t
-      // with t = (S_M - u) / den, exactly 1 where S_M = u
-      const R t = (sm - ul) * (R(1) / denl);
-      fv = bn * t;
-      fb = R(1) + rsl * t;
-    } else {
-      fv = bn * (sm - ul) / denl;
-      fb = (rsl * sdl - bn2) / denl;
-    }
+    // numerator of fb = den + rho (S - u)(S_M - u): fb = 1 + rho (S - u) t
+    // with t = (S_M - u) / den, exactly 1 where S_M = u
+    const R t = (sm - ul) * (R(1) / denl);
+    const R fv = bn * t, fb = R(1) + rsl * t;
     vls = vl - byl * fv; wls = wl_ - bzl * fv;
     byls = byl * fb; bzls = bzl * fb;
   }
@@ -222,17 +273,10 @@ __device__ __forceinline__ void hlld(const R* L, const R* Rr, R bn, R gamma, R i
   if (Tr<R>::abs(denr) <= Tr<R>::degen() * rmax(rsr * sdr, bn2)) {
     vrs = vr; wrs = wr_; byrs = byr; bzrs = bzr;
   } else {
-    R fv, fb;
-    if constexpr (FR) {
-      // numerator of fb = den + rho (S - u)(S_M - u): fb = 1 + rho (S - u) t
-      // with t = (S_M - u) / den, exactly 1 where S_M = u
-      const R t = (sm - ur) * (R(1) / denr);
-      fv = bn * t;
-      fb = R(1) + rsr * t;
-    } else {
-      fv = bn * (sm - ur) / denr;
-      fb = (rsr * sdr - bn2) / denr;
-    }
+    // numerator of fb = den + rho (S - u)(S_M - u): fb = 1 + rho (S - u) t
+    // with t = (S_M - u) / den, exactly 1 where S_M = u
+    const R t = (sm - ur) * (R(1) / denr);
+    const R fv = bn * t, fb = R(1) + rsr * t;
     vrs = vr - byr * fv; wrs = wr_ - bzr * fv;
     byrs = byr * fb; bzrs = bzr * fb;
   }
@@ -240,22 +284,12 @@ __device__ __forceinline__ void hlld(const R* L, const R* Rr, R bn, R gamma, R i
   R vbr = ur * bn + vr * byr + wr_ * bzr;
   R vbls = sm * bn + vls * byls + wls * bzls;
   R vbrs = sm * bn + vrs * byrs + wrs * bzrs;
-  R els = qdiv<FR>(((sdl * el - ptl * ul) + pts * sm) + bn * (vbl - vbls), sml, isml);
-  R ers = qdiv<FR>(((sdr * er - ptr * ur) + pts * sm) + bn * (vbr - vbrs), smr, ismr);
+  R els = (((sdl * el - ptl * ul) + pts * sm) + bn * (vbl - vbls)) * isml;
+  R ers = (((sdr * er - ptr * ur) + pts * sm) + bn * (vbr - vbrs)) * ismr;
 
-  R sqrl, sqrr, sls, srs;
-  if constexpr (FR) {
-    const R isl = Tr<R>::rsqrt_(rls), isr = Tr<R>::rsqrt_(rrs);
-    sqrl = rls * isl;
-    sqrr = rrs * isr;
-    sls = sm - Tr<R>::abs(bn) * isl;
-    srs = sm + Tr<R>::abs(bn) * isr;
-  } else {
-    sqrl = Tr<R>::sqrt_(rls);
-    sqrr = Tr<R>::sqrt_(rrs);
-    sls = sm - Tr<R>::abs(bn) / sqrl;
-    srs = sm + Tr<R>::abs(bn) / sqrr;
-  }
+  const R isl = Tr<R>::rsqrt_(rls), isr = Tr<R>::rsqrt_(rrs);
+  const R sqrl = rls * isl, sqrr = rrs * isr;
+  const R sls = sm - Tr<R>::abs(bn) * isl, srs = sm + Tr<R>::abs(bn) * isr;
 
   R fo[8];
   if (sls >= R(0) || srs < R(0)) {
@@ -276,11 +310,11 @@ __device__ __forceinline__ void hlld(const R* L, const R* Rr, R bn, R gamma, R i
 
   R sgn = (bn >= R(0)) ? R(1) : R(-1);
   R ssum = sqrl + sqrr;
-  const R iss = recip<FR>(ssum);
-  R vss = qdiv<FR>((sqrl * vls + sqrr * vrs) + sgn * (byrs - byls), ssum, iss);
-  R wss = qdiv<FR>((sqrl * wls + sqrr * wrs) + sgn * (bzrs - bzls), ssum, iss);
-  R byss = qdiv<FR>((sqrl * byrs + sqrr * byls) + sgn * (sqrl * sqrr) * (vrs - vls), ssum, iss);
-  R bzss = qdiv<FR>((sqrl * bzrs + sqrr * bzls) + sgn * (sqrl * sqrr) * (wrs - wls), ssum, iss);
+  const R iss = R(1) / ssum;
+  R vss = ((sqrl * vls + sqrr * vrs) + sgn * (byrs - byls)) * iss;
+  R wss = ((sqrl * wls + sqrr * wrs) + sgn * (bzrs - bzls)) * iss;
+  R byss = ((sqrl * byrs + sqrr * byls) + sgn * (sqrl * sqrr) * (vrs - vls)) * iss;
+  R bzss = ((sqrl * bzrs + sqrr * bzls) + sgn * (sqrl * sqrr) * (wrs - wls)) * iss;
   R vbss = sm * bn + vss * byss + wss * bzss;
 
   const bool left = (sm >= R(0));
@@ -301,6 +335,207 @@ __device__ __forceinline__ void hlld(const R* L, const R* Rr, R bn, R gamma, R i
     R fs = fo[q] + S * (us[q] - u0[q]);
     f[q] = fs + Ss * (uss[q] - us[q]);
   }
+}
+
+// HLLD flux (Miyoshi & Kusano 2005) between rotated primitive states L (lower
+// side) and R_ (upper side) with interface normal field bn.  Wave speeds
+// S_L = min(u_L,u_R) - max(cf), S_R = max(u_L,u_R) + max(cf); S_M, p_T* from
+// MK05 eqs. (38), (41); star states eqs. (43)-(48) with a degenerate branch
+// (|rho(S-u)(S-S_M) - Bn^2| <= degen max(rho(S-u)^2, Bn^2), degen 1e-12 in
+// FP64 and 1e-5 in FP32, keeps the outer
+// transverse v, B); Alfven speeds S* = S_M -/+ |Bn|/sqrt(rho*); double-star
+// states eqs. (59)-(63); left-closed region selection.  f gets the rotated
+// flux (f[5], the normal-B component, is 0); *upw, where up is set (the
+// upwinded EMF average), the upwind side of the contact (+1, -1, or 0 when
+// |S_M| <= eps_up (S_R - S_L)), else 0.
+// The interface lies in the half of the fan on S_M's side (S_M >= 0: left):
+// a star region left of the contact needs S*_L <= S_M, one right of it
+// S_M <= S*_R.  So the energies, the Alfven speed and the flux are computed
+// for that side alone, from operands selected first, with the expressions
+// (and in the parity build the bits) they would have on either side; only the
+// transverse star states, which the double-star states mix, are computed for
+// both.
+// FR: quotients with a common denominator multiply by its reciprocal (8
+// divisions per face instead of 16), and the single-star field factor
+// is written as 1 + rho (S - u)(S_M - u)/den, which is exactly 1 where
+// S_M = u (a plain reciprocal would turn x/x into x (1/x), off by an ulp,
+// and give a 2D problem a z-field of rounding noise).
+template <typename R, bool FR = false>
+__device__ __forceinline__ void hlld64(const R* L, const R* Rr, R bn, R gamma, R igm1, R eps_up, bool up,
+                                     R* f, R* upw) {
+  using T = Tr<R>;
+  R rl = L[0], ul = L[1], vl = L[2], wl_ = L[3], pl = L[4], byl = L[6], bzl = L[7];
+  R rr = Rr[0], ur = Rr[1], vr = Rr[2], wr_ = Rr[3], pr = Rr[4], byr = Rr[6], bzr = Rr[7];
+
+  R cfl = fast_speed(rl, pl, bn, byl, bzl, gamma);
+  R cfr = fast_speed(rr, pr, bn, byr, bzr, gamma);
+  R cmax = T::less_mag(cfr, cfl) ? cfl : cfr;
+  const bool ulo = ul < ur;
+  R sl = (ulo ? ul : ur) - cmax;
+  R sr = (ulo ? ur : ul) + cmax;
+
+  if (T::ge0(sl)) {
+    flux_rot(L, bn, igm1, f);
+    *upw = R(1);
+    return;
+  }
+  if (T::neg(sr)) {
+    flux_rot(Rr, bn, igm1, f);
+    *upw = R(-1);
+    return;
+  }
+
+  R pml = T::half(bn * bn + byl * byl + bzl * bzl);
+  R pmr = T::half(bn * bn + byr * byr + bzr * bzr);
+  R ptl = pl + pml, ptr = pr + pmr;
+  R sdl = sl - ul, sdr = sr - ur;
+  R rsl = sdl * rl, rsr = sdr * rr;
+  R dd = rsr - rsl;
+  const R idd = recip<FR>(dd);
+  R sm = qdiv<FR>((rsr * ur - rsl * ul) - (ptr - ptl), dd, idd);
+  *upw = R(0);
+  if (up && T::abs_gt(sm, eps_up * (sr - sl))) *upw = T::neg(sm) ? R(-1) : R(1);
+
+  R sml = sl - sm, smr = sr - sm;
+  const R isml = recip<FR>(sml), ismr = recip<FR>(smr);
+  R rls = qdiv<FR>(rsl, sml, isml), rrs = qdiv<FR>(rsr, smr, ismr);
+  R bn2 = bn * bn;
+  R vls, wls, byls, bzls;
+  R denl = rsl * sml - bn2;
+  const bool dgl = T::degenerate(denl, rsl, sdl, bn2);
+  if (dgl) {
+    vls = vl; wls = wl_; byls = byl; bzls = bzl;
+  } else {
+    R fv, fb;
+    if constexpr (FR) {
+      // numerator of fb = den + rho (S - u)(S_M - u): fb = 1 + rho (S - u) t
+      // with t = (S_M - u) / den, exactly 1 where S_M = u
+      const R t = (sm - ul) * recip<FR>(denl);
+      fv = bn * t;
+      fb = R(1) + rsl * t;
+    } else {
+      fv = T::div(bn * (sm - ul), denl);
+      fb = T::div(rsl * sdl - bn2, denl);
+    }
+    vls = vl - byl * fv; wls = wl_ - bzl * fv;
+    byls = byl * fb; bzls = bzl * fb;
+  }
+  R vrs, wrs, byrs, bzrs;
+  R denr = rsr * smr - bn2;
+  const bool dgr = T::degenerate(denr, rsr, sdr, bn2);
+  if (dgr) {
+    vrs = vr; wrs = wr_; byrs = byr; bzrs = bzr;
+  } else {
+    R fv, fb;
+    if constexpr (FR) {
+      const R t = (sm - ur) * recip<FR>(denr);
+      fv = bn * t;
+      fb = R(1) + rsr * t;
+    } else {
+      fv = T::div(bn * (sm - ur), denr);
+      fb = T::div(rsr * sdr - bn2, denr);
+    }
+    vrs = vr - byr * fv; wrs = wr_ - bzr * fv;
+    byrs = byr * fb; bzrs = bzr * fb;
+  }
+
+  // the side of the contact the interface lies on
+  const bool left = T::ge0(sm);
+  const R rho = left ? rl : rr, u = left ? ul : ur, v = left ? vl : vr, w = left ? wl_ : wr_;
+  const R p = left ? pl : pr, by = left ? byl : byr, bz = left ? bzl : bzr;
+  const R pm = left ? pml : pmr, pt = left ? ptl : ptr;
+  // p_T*: MK05 eq. (41), or FR eq. (23) on the selected side, p_T + rho (S - u)
+  // (S_M - u), which is exactly p_T in a uniform state
+  R pts;
+  if constexpr (FR) pts = pt + (left ? rsl : rsr) * (sm - u);
+  else pts = T::div((rsr * ptl - rsl * ptr) + rsl * rsr * (ur - ul), dd);
+  const R S = left ? sl : sr, sd = left ? sdl : sdr, sS = left ? sml : smr, isS = left ? isml : ismr;
+  const R rs = left ? rls : rrs, vs = left ? vls : vrs, ws = left ? wls : wrs;
+  const R bys = left ? byls : byrs, bzs = left ? bzls : bzrs;
+  const R e = p * igm1 + T::half(rho) * (u * u + v * v + w * w) + pm;
+  const R vb = u * bn + v * by + w * bz;
+  const R vbs = sm * bn + vs * bys + ws * bzs;
+  const R es = qdiv<FR>(((sd * e - pt * u) + pts * sm) + bn * (vb - vbs), sS, isS);
+
+  R sqrl, sqrr, ab;
+  sqrl = T::sqrt_(rls);
+  sqrr = T::sqrt_(rrs);
+  ab = T::div(T::abs(bn), left ? sqrl : sqrr);
+  const R Ss = left ? sm - ab : sm + ab;
+
+  const R mxs = rs * sm;
+  const bool bneg = !T::ge0(bn);
+  const bool single = left ? T::ge0(Ss) : T::neg(Ss);
+  if constexpr (FR) {
+    // F* = F + S (U* - U) and F** = F* + S* (U** - U*) are the physical fluxes
+    // of the star states (pressure p_T*, normal velocity S_M), the jumps being
+    // the Rankine-Hugoniot conditions that define those states: one flux of
+    // the state the interface lies in, 14 operations instead of 42.  A
+    // degenerate outer state kept its transverse field, whose induction flux
+    // then moves with the outer velocity.
+    R vF = vs, wF = ws, byF = bys, bzF = bzs, eF = es, vbF = vbs;
+    if (!single) {
+      // the double-star state as changes from the side's star state, which
+      // vanish exactly in a uniform state: dv = (sqrt(rho*) of the other side
+      // times the velocity jump, plus the field jump) / sum, dB = sqrt(rho*) dv
+      const R iss = recip<FR>(sqrl + sqrr), so = left ? sqrr : sqrl, ss = left ? sqrl : sqrr;
+      const R dv = (flip(so * (vrs - vls), !left) + flip(byrs - byls, bneg)) * iss;
+      const R dw = (flip(so * (wrs - wls), !left) + flip(bzrs - bzls, bneg)) * iss;
+      vF = vs + dv;
+      wF = ws + dw;
+      byF = bys + flip(ss * dv, left == bneg);
+      bzF = bzs + flip(ss * dw, left == bneg);
+      vbF = sm * bn + vF * byF + wF * bzF;
+      eF = es + flip(ss * (vbs - vbF), left != bneg);
+    }
+    f[0] = mxs;
+    f[1] = mxs * sm + (pts - bn2);
+    f[2] = mxs * vF - bn * byF;
+    f[3] = mxs * wF - bn * bzF;
+    f[4] = (eF + pts) * sm - bn * vbF;
+    f[5] = R(0);
+    f[6] = byF * sm - bn * vF;
+    f[7] = bzF * sm - bn * wF;
+    if (left ? dgl : dgr) {
+      f[6] = f[6] + bys * (u - sm);
+      f[7] = f[7] + bzs * (u - sm);
+    }
+    return;
+  }
+  // outer flux and conserved states; single-star region: F* = F + S (U* - U)
+  const R mx = rho * u, my = rho * v, mz = rho * w;
+  const R mys = rs * vs, mzs = rs * ws;
+  f[0] = mx + S * (rs - rho);
+  f[1] = (mx * u + pt - bn2) + S * (mxs - mx);
+  f[2] = (mx * v - bn * by) + S * (mys - my);
+  f[3] = (mx * w - bn * bz) + S * (mzs - mz);
+  f[4] = ((e + pt) * u - bn * vb) + S * (es - e);
+  f[5] = R(0);
+  f[6] = (by * u - bn * v) + S * (bys - by);
+  f[7] = (bz * u - bn * w) + S * (bzs - bz);
+  if (single) return;
+
+  // double-star region: F** = F* + S* (U** - U*); rho and S_M are U*'s
+  R ssum = sqrl + sqrr;
+  R vss = T::div((sqrl * vls + sqrr * vrs) + flip(byrs - byls, bneg), ssum);
+  R wss = T::div((sqrl * wls + sqrr * wrs) + flip(bzrs - bzls, bneg), ssum);
+  const R sq2 = flip(sqrl * sqrr, bneg);
+  R byss = T::div((sqrl * byrs + sqrr * byls) + sq2 * (vrs - vls), ssum);
+  R bzss = T::div((sqrl * bzrs + sqrr * bzls) + sq2 * (wrs - wls), ssum);
+  R vbss = sm * bn + vss * byss + wss * bzss;
+  const R ess = es + flip((left ? sqrl : sqrr) * (vbs - vbss), left != bneg);
+  f[2] = f[2] + Ss * (rs * vss - mys);
+  f[3] = f[3] + Ss * (rs * wss - mzs);
+  f[4] = f[4] + Ss * (ess - es);
+  f[6] = f[6] + Ss * (byss - bys);
+  f[7] = f[7] + Ss * (bzss - bzs);
+}
+
+template <typename R, bool FR = false>
+__device__ __forceinline__ void hlld(const R* L, const R* Rr, R bn, R gamma, R igm1, R eps_up, bool up, R* f,
+                                     R* upw) {
+  if constexpr (sizeof(R) == 4) hlld32(L, Rr, bn, gamma, igm1, eps_up, f, upw);
+  else hlld64<R, FR>(L, Rr, bn, gamma, igm1, eps_up, up, f, upw);
 }
 
 }  // namespace mhd
