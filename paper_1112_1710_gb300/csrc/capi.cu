@@ -23,23 +23,48 @@ using namespace mhd;
 
 namespace {
 
-// A device copy of a small host table, keyed by its bytes.  Entries are
+// A device copy of a host table, found by a key: the table's own bytes, or the
+// (much shorter) sizes it is built from.  Entries are
 // immutable once uploaded, so a launch may still be reading one while the
 // host prepares the next call; repeated calls with the same descriptors
-// (every step of a static hierarchy) upload nothing.
+// (every step of a static hierarchy) build and upload nothing.
 struct TableEntry {
-  std::vector<char> bytes;
+  std::vector<char> key;
+  int kind = 0;       // what the key describes (TableKind)
   void* dev = nullptr;
+  size_t count = 0;   // elements of the table
 };
 
-uint64_t fnv1a(const void* p, size_t n) {
+enum TableKind : int {
+  TK_BYTES = 0,       // the table itself
+  TK_TASKS,           // element counts -> blocks (tasks_for)
+  TK_REGION2, TK_REGION1, TK_REGIONU,  // patch sizes -> blocks of an advance stage
+  TK_PRED_TILES,      // patch sizes -> tiles of the tiled predictor
+  TK_PF_ITEMS,        // patch sizes, tile and chunk -> fused pass items
+  TK_FUSED_ITEMS, TK_FUSED_TASKS,      // the same for the fused kernel
+  TK_PACKED, TK_STARTS,                // element counts -> packed blocks, first elements
+  TK_GHOST_COPIES, TK_GHOST_EXCL, TK_GHOST_TASKS64, TK_GHOST_TASKS32  // copies -> the ghost fill's tables
+};
+
+// Hash of n bytes, eight at a time on four chains (a multiplication's latency
+// per 32 bytes; a byte-wise hash of an advance's tables took longer on the
+// host than the advance of a million cells on the GPU).
+uint64_t hash_bytes(int kind, const void* p, size_t n) {
   const unsigned char* c = (const unsigned char*)p;
-  uint64_t h = 1469598103934665603ULL;
-  for (size_t i = 0; i < n; ++i) {
-    h ^= c[i];
-    h *= 1099511628211ULL;
-  }
-  return h;
+  const uint64_t K = 0x9E3779B97F4A7C15ull;
+  uint64_t h[4] = {K ^ (uint64_t)kind, K + 1, K + 2, K + n};
+  size_t i = 0;
+  for (; i + 32 <= n; i += 32)
+    for (int k = 0; k < 4; ++k) {
+      uint64_t w;
+      std::memcpy(&w, c + i + 8 * k, 8);
+      h[k] = (h[k] ^ w) * K;
+      h[k] ^= h[k] >> 29;
+    }
+  uint64_t r = h[0];
+  for (int k = 1; k < 4; ++k) r = (r ^ h[k]) * K, r ^= r >> 31;
+  for (; i < n; ++i) r = (r ^ c[i]) * K, r ^= r >> 32;
+  return r;
 }
 
 }  // namespace
@@ -99,42 +124,56 @@ mhd_status cuda_fail(mhd_ctx* c, cudaError_t e, const char* what) {
   return fail(c, MHD_ECUDA, "%s: %s", what, cudaGetErrorString(e));
 }
 
-// Returns a device pointer holding `n` bytes equal to `host`.
-mhd_status table(mhd_ctx* c, const void* host, size_t n, void** out) {
-  if (n == 0) {
-    *out = nullptr;
-    return MHD_OK;
-  }
-  const uint64_t h = fnv1a(host, n);
+// The table of kind `kind` whose key is the nkey bytes at `key`: the cached one,
+// or what `build` appends to an empty vector, uploaded.
+template <typename T, typename Build>
+mhd_status keyed_table(mhd_ctx* c, int kind, const void* key, size_t nkey, Build build, const T** out, int* count) {
+  const uint64_t h = hash_bytes(kind, key, nkey);
   auto range = c->tables.equal_range(h);
   for (auto it = range.first; it != range.second; ++it) {
-    if (it->second.bytes.size() == n && std::memcmp(it->second.bytes.data(), host, n) == 0) {
-      *out = it->second.dev;
+    const TableEntry& e = it->second;
+    if (e.kind == kind && e.key.size() == nkey && (nkey == 0 || std::memcmp(e.key.data(), key, nkey) == 0)) {
+      *out = (const T*)e.dev;
+      *count = (int)e.count;
       return MHD_OK;
     }
   }
-  if (c->table_bytes + n > kTableCacheLimit) {
-    // drop every cached table; launches in flight may still read them
-    cudaError_t e = cudaDeviceSynchronize();
-    if (e != cudaSuccess) return cuda_fail(c, e, "table cache flush");
-    for (auto& kv : c->tables) cudaFree(kv.second.dev);
-    c->tables.clear();
-    c->table_bytes = 0;
-  }
+  std::vector<T> v;
+  build(v);
+  if (v.size() > 0x7fffffff) return fail(c, MHD_EINVAL, "launch too large");
   TableEntry t;
-  t.bytes.assign((const char*)host, (const char*)host + n);
-  cudaError_t e = cudaMalloc(&t.dev, n);
-  if (e != cudaSuccess) return fail(c, MHD_ENOMEM, "table alloc of %zu bytes: %s", n, cudaGetErrorString(e));
-  // synchronous copy: the entry is immutable from here on
-  e = cudaMemcpy(t.dev, host, n, cudaMemcpyHostToDevice);
-  if (e != cudaSuccess) {
-    cudaFree(t.dev);
-    return cuda_fail(c, e, "table upload");
+  t.kind = kind;
+  t.key.assign((const char*)key, (const char*)key + nkey);
+  t.count = v.size();
+  const size_t n = v.size() * sizeof(T);
+  if (n > 0) {
+    cudaError_t e = cudaMalloc(&t.dev, n);
+    if (e != cudaSuccess) return fail(c, MHD_ENOMEM, "table alloc of %zu bytes: %s", n, cudaGetErrorString(e));
+    // synchronous copy: the entry is immutable from here on
+    e = cudaMemcpy(t.dev, v.data(), n, cudaMemcpyHostToDevice);
+    if (e != cudaSuccess) {
+      cudaFree(t.dev);
+      return cuda_fail(c, e, "table upload");
+    }
   }
-  *out = t.dev;
-  c->table_bytes += n;
+  *out = (const T*)t.dev;
+  *count = (int)t.count;
+  c->table_bytes += n + nkey;
   c->tables.emplace(h, std::move(t));
   return MHD_OK;
+}
+
+// Returns a device pointer holding `n` bytes equal to `host`.
+mhd_status table(mhd_ctx* c, const void* host, size_t n, void** out) {
+  *out = nullptr;
+  if (n == 0) return MHD_OK;
+  const char* dev = nullptr;
+  int count = 0;
+  mhd_status r = keyed_table<char>(
+      c, TK_BYTES, host, n, [&](std::vector<char>& v) { v.assign((const char*)host, (const char*)host + n); }, &dev,
+      &count);
+  *out = const_cast<char*>(dev);
+  return r;
 }
 
 mhd_status ensure_scratch(mhd_ctx* c, size_t bytes) {
@@ -222,6 +261,16 @@ mhd_status begin(mhd_ctx* c) {
   if (!c) return MHD_EINVAL;
   cudaError_t e = cudaSetDevice(c->device);
   if (e != cudaSuccess) return cuda_fail(c, e, "cudaSetDevice");
+  if (c->table_bytes > kTableCacheLimit) {
+    // drop every cached table, between calls (a call's own tables stay);
+    // launches in flight may still read them
+    e = cudaDeviceSynchronize();
+    if (e != cudaSuccess) return cuda_fail(c, e, "table cache flush");
+    for (auto& kv : c->tables)
+      if (kv.second.dev) cudaFree(kv.second.dev);
+    c->tables.clear();
+    c->table_bytes = 0;
+  }
   return MHD_OK;
 }
 
@@ -240,29 +289,37 @@ void tasks_for(const std::vector<int64_t>& counts, std::vector<BlockTask>& out) 
 // flux-register captures), where threads of one block then read different
 // items.
 mhd_status packed_table(mhd_ctx* c, const std::vector<int64_t>& counts, bool packed, PackedTasks& out) {
-  std::vector<int64_t> starts(counts.size() + 1, 0);
-  for (size_t i = 0; i < counts.size(); ++i) starts[i + 1] = starts[i] + counts[i];
-  std::vector<BlockTask> tasks;
-  if (packed) {
-    size_t item = 0;
-    for (int64_t b = 0; b < starts.back(); b += kThreads) {
-      while (starts[item + 1] <= b) ++item;
-      tasks.push_back(BlockTask{(int32_t)item, (int32_t)(b - starts[item])});
-    }
-  } else {
-    tasks_for(counts, tasks);
-  }
-  if (tasks.size() > 0x7fffffff || counts.size() > 0x7fffffff) return fail(c, MHD_EINVAL, "launch too large");
-  void *d_t = nullptr, *d_s = nullptr;
-  mhd_status r = table(c, tasks.data(), tasks.size() * sizeof(BlockTask), &d_t);
-  if (!r) r = table(c, starts.data(), starts.size() * sizeof(int64_t), &d_s);
+  auto starts_of = [&](std::vector<int64_t>& starts) {
+    starts.assign(counts.size() + 1, 0);
+    for (size_t i = 0; i < counts.size(); ++i) starts[i + 1] = starts[i] + counts[i];
+  };
+  const size_t nkey = counts.size() * sizeof(int64_t);
+  int n = 0;
+  mhd_status r = keyed_table<BlockTask>(
+      c, packed ? TK_PACKED : TK_TASKS, counts.data(), nkey,
+      [&](std::vector<BlockTask>& tasks) {
+        if (!packed) return tasks_for(counts, tasks);
+        std::vector<int64_t> starts;
+        starts_of(starts);
+        size_t item = 0;
+        for (int64_t b = 0; b < starts.back(); b += kThreads) {
+          while (starts[item + 1] <= b) ++item;
+          tasks.push_back(BlockTask{(int32_t)item, (int32_t)(b - starts[item])});
+        }
+      },
+      &out.tasks, &out.nblocks);
+  if (!r) r = keyed_table<int64_t>(c, TK_STARTS, counts.data(), nkey, starts_of, &out.starts, &n);
   if (r) return r;
-  out.tasks = (const BlockTask*)d_t;
-  out.starts = (const int64_t*)d_s;
-  out.nblocks = (int)tasks.size();
   out.nitems = (int)counts.size();
   out.packed = packed ? 1 : 0;
   return MHD_OK;
+}
+
+// The blocks of tasks_for on the device.
+mhd_status tasks_table(mhd_ctx* c, const std::vector<int64_t>& counts, const BlockTask** out, int* nblocks) {
+  return keyed_table<BlockTask>(
+      c, TK_TASKS, counts.data(), counts.size() * sizeof(int64_t),
+      [&](std::vector<BlockTask>& v) { tasks_for(counts, v); }, out, nblocks);
 }
 
 // Counts of the top-layer items (box i, axis a) -> item 3 i + a: the box's
@@ -275,29 +332,42 @@ std::vector<int64_t> top_counts(const std::vector<std::array<int32_t, 3>>& ext) 
   return out;
 }
 
-// Block tables of the staged advance: over each patch's UB+2 (t2), the
-// predictor / flux region (t1) and the update region (tu) of an element of
-// `elem` bytes; UB = interior grown by the patch's k.
-void staged_tasks(const std::vector<DPatch>& dp, size_t elem, std::vector<BlockTask>& t2,
-                  std::vector<BlockTask>& t1, std::vector<BlockTask>& tu) {
-  const size_t n = dp.size();
-  const int m1 = region_m1(elem), mu = region_mu(elem) + region_mu_top(elem);
-  std::vector<int64_t> c2(n), c1(n), cu(n);
-  for (size_t p = 0; p < n; ++p) {
-    int64_t v2 = 1, v1 = 1, vu = 1;
-    for (int d = 0; d < 3; ++d) {
-      const int64_t e = dp[p].n[d] + 2 * dp[p].k;
-      v2 *= e + 4;
-      v1 *= e + 2 * m1;
-      vu *= e + mu;
-    }
-    c2[p] = v2;
-    c1[p] = v1;
-    cu[p] = vu;
-  }
-  tasks_for(c2, t2);
-  tasks_for(c1, t1);
-  tasks_for(cu, tu);
+// What the block tables of an advance depend on, per patch.
+struct PatchSize {
+  int32_t n[3], g, k;
+};
+std::vector<PatchSize> sizes_of(const std::vector<DPatch>& dp) {
+  std::vector<PatchSize> out(dp.size());
+  for (size_t p = 0; p < dp.size(); ++p) out[p] = PatchSize{{dp[p].n[0], dp[p].n[1], dp[p].n[2]}, dp[p].g, dp[p].k};
+  return out;
+}
+
+// Block table of one region of the staged advance: the update box UB (interior
+// grown by k) of each patch with `grow` more cells along each axis: UB+2
+// (kind TK_REGION2), the predictor / flux region (TK_REGION1), the update
+// region (TK_REGIONU).
+mhd_status region_table(mhd_ctx* c, int kind, int grow, const std::vector<PatchSize>& ps, const BlockTask** out,
+                        int* nblocks) {
+  return keyed_table<BlockTask>(
+      c, kind, ps.data(), ps.size() * sizeof(PatchSize),
+      [&](std::vector<BlockTask>& v) {
+        std::vector<int64_t> cnt(ps.size());
+        for (size_t p = 0; p < ps.size(); ++p) {
+          cnt[p] = 1;
+          for (int d = 0; d < 3; ++d) cnt[p] *= ps[p].n[d] + 2 * ps[p].k + grow;
+        }
+        tasks_for(cnt, v);
+      },
+      out, nblocks);
+}
+
+// The staged advance's block tables into its arguments (`all`: the update
+// region's only otherwise).
+mhd_status staged_tables(mhd_ctx* c, const std::vector<PatchSize>& ps, size_t elem, bool all, AdvanceArgs& a) {
+  mhd_status r = region_table(c, TK_REGIONU, region_mu(elem) + region_mu_top(elem), ps, &a.tasksu, &a.nblocksu);
+  if (!r && all) r = region_table(c, TK_REGION2, 4, ps, &a.tasks, &a.nblocks);
+  if (!r && all) r = region_table(c, TK_REGION1, 2 * region_m1(elem), ps, &a.tasks1, &a.nblocks1);
+  return r;
 }
 
 double eps_for(const mhd_params& prm, int dtype) {
@@ -400,7 +470,8 @@ void mhd_ctx_destroy(mhd_ctx* c) {
   if (!c) return;
   cudaSetDevice(c->device);
   cudaDeviceSynchronize();
-  for (auto& kv : c->tables) cudaFree(kv.second.dev);
+  for (auto& kv : c->tables)
+    if (kv.second.dev) cudaFree(kv.second.dev);
   if (c->scratch) cudaFree(c->scratch);
   if (c->partials) cudaFree(c->partials);
   if (c->d_status) cudaFree(c->d_status);
@@ -585,6 +656,45 @@ void pred_tiles(const std::vector<DPatch>& dp, int dtype, std::vector<BlockTask>
   }
 }
 
+// Key of a table built from the patches' sizes and a few parameters.
+std::vector<int32_t> sized_key(const std::vector<PatchSize>& ps, std::initializer_list<int32_t> prm) {
+  std::vector<int32_t> key(prm);
+  const int32_t* q = (const int32_t*)ps.data();
+  key.insert(key.end(), q, q + ps.size() * (sizeof(PatchSize) / sizeof(int32_t)));
+  return key;
+}
+
+mhd_status pf_table(mhd_ctx* c, const std::vector<DPatch>& dp, const std::vector<PatchSize>& ps, const PfVariant& v,
+                    int cz, AdvanceArgs& a) {
+  const std::vector<int32_t> key = sized_key(ps, {v.tx, v.ty, cz});
+  return keyed_table<FusedItem>(
+      c, TK_PF_ITEMS, key.data(), key.size() * sizeof(int32_t),
+      [&](std::vector<FusedItem>& items) { pf_items(dp, v.tx, v.ty, cz, items); }, &a.pf_items, &a.npf);
+}
+
+mhd_status fused_tables(mhd_ctx* c, const std::vector<DPatch>& dp, const std::vector<PatchSize>& ps,
+                        const FusedVariant& v, int cz, AdvanceArgs& a) {
+  const std::vector<int32_t> key = sized_key(ps, {v.bx, v.by, cz});
+  std::vector<FusedItem> items;
+  std::vector<BlockTask> ctasks;
+  mhd_status r = keyed_table<FusedItem>(
+      c, TK_FUSED_ITEMS, key.data(), key.size() * sizeof(int32_t),
+      [&](std::vector<FusedItem>& out) { fused_items(dp, v.bx, v.by, cz, out, ctasks); }, &a.items, &a.nitems);
+  if (!r)
+    r = keyed_table<BlockTask>(
+        c, TK_FUSED_TASKS, key.data(), key.size() * sizeof(int32_t),
+        [&](std::vector<BlockTask>& out) { fused_items(dp, v.bx, v.by, cz, items, out); }, &a.ctasks, &a.nctasks);
+  return r;
+}
+
+mhd_status pred_table(mhd_ctx* c, const std::vector<DPatch>& dp, const std::vector<PatchSize>& ps, int dtype,
+                      AdvanceArgs& a) {
+  const std::vector<int32_t> key = sized_key(ps, {dtype});
+  return keyed_table<BlockTask>(
+      c, TK_PRED_TILES, key.data(), key.size() * sizeof(int32_t),
+      [&](std::vector<BlockTask>& out) { pred_tiles(dp, dtype, out); }, &a.ptasks, &a.npblocks);
+}
+
 int sm_count(int dev) {
   int nsm = 0;
   if (cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || nsm < 1) nsm = 1;
@@ -708,51 +818,31 @@ static mhd_status advance_impl(mhd_ctx* c, const mhd_patch_desc* patches, int32_
   const size_t es = elem_size(dtype);
   const size_t counter_byte = ((size_t)off * es + 15) / 16 * 16;
   if ((r = ensure_scratch(c, counter_byte + 16))) return r;
-  std::vector<BlockTask> tasks, tasks1, tasksu, ptasks;
-  std::vector<FusedItem> items;
-  std::vector<BlockTask> ctasks;
   const int di = dtype == MHD_F32 ? 1 : 0;
   const int shape = c->prm.kernel_shape > 0 ? c->prm.kernel_shape - 1 : pf ? c->pf_variant[di] : c->fused_variant[di];
   if (shape >= (pf ? (di ? kNumPf32 : kNumPf64) : (di ? kNumFused32 : kNumFused64)))
     return fail(c, MHD_EINVAL, "kernel_shape %d is not compiled for this element type", c->prm.kernel_shape);
+  AdvanceArgs a{};
+  const std::vector<PatchSize> ps = sizes_of(dp);
   if (pf) {
-    staged_tasks(dp, elem_size(dtype), tasks, tasks1, tasksu);
-    const PfVariant& pv = di ? kPfVariants32[shape] : kPfVariants64[shape];
-    pf_items(dp, pv.tx, pv.ty,
-             c->prm.fused_chunk > 0 ? c->prm.fused_chunk : c->fused_chunk[di] > 0 ? c->fused_chunk[di] : 16, items);
-    if (items.size() > 0x7fffffff || tasksu.size() > 0x7fffffff) return fail(c, MHD_EINVAL, "launch too large");
+    const int cz = c->prm.fused_chunk > 0 ? c->prm.fused_chunk : c->fused_chunk[di] > 0 ? c->fused_chunk[di] : 16;
+    if ((r = staged_tables(c, ps, es, false, a))) return r;
+    if ((r = pf_table(c, dp, ps, di ? kPfVariants32[shape] : kPfVariants64[shape], cz, a))) return r;
   } else if (!fused) {
-    staged_tasks(dp, elem_size(dtype), tasks, tasks1, tasksu);
-    if (c->prm.advance_kernel == 3 || c->pred_tiled[dtype == MHD_F32 ? 1 : 0]) pred_tiles(dp, dtype, ptasks);
-    if (tasks.size() > 0x7fffffff || ptasks.size() > 0x7fffffff) return fail(c, MHD_EINVAL, "launch too large");
+    if ((r = staged_tables(c, ps, es, true, a))) return r;
+    if (c->prm.advance_kernel == 3 || c->pred_tiled[di])
+      if ((r = pred_table(c, dp, ps, dtype, a))) return r;
   } else {
     const FusedVariant& v = fused_variant_of(dtype, shape);
     const int cz = c->prm.fused_chunk > 0   ? c->prm.fused_chunk
                    : c->fused_chunk[di] > 0 ? c->fused_chunk[di]
                                             : fused_chunk_auto(dp, v.bx, v.by, sm_count(c->device));
-    fused_items(dp, v.bx, v.by, cz, items, ctasks);
-    if (items.size() > 0x7fffffff) return fail(c, MHD_EINVAL, "launch too large");
+    if ((r = fused_tables(c, dp, ps, v, cz, a))) return r;
   }
-  void *d_p = nullptr, *d_t = nullptr, *d_t1 = nullptr, *d_tu = nullptr, *d_i = nullptr, *d_ct = nullptr,
-       *d_pt = nullptr;
+  void* d_p = nullptr;
   if ((r = table(c, dp.data(), dp.size() * sizeof(DPatch), &d_p))) return r;
-  if ((r = table(c, tasks.data(), tasks.size() * sizeof(BlockTask), &d_t))) return r;
-  if ((r = table(c, tasks1.data(), tasks1.size() * sizeof(BlockTask), &d_t1))) return r;
-  if ((r = table(c, tasksu.data(), tasksu.size() * sizeof(BlockTask), &d_tu))) return r;
-  if ((r = table(c, ptasks.data(), ptasks.size() * sizeof(BlockTask), &d_pt))) return r;
-  if ((r = table(c, items.data(), items.size() * sizeof(FusedItem), &d_i))) return r;
-  if ((r = table(c, ctasks.data(), ctasks.size() * sizeof(BlockTask), &d_ct))) return r;
-  AdvanceArgs a{};
   a.patches = (const DPatch*)d_p;
   a.npatches = n;
-  a.tasks = (const BlockTask*)d_t;
-  a.nblocks = (int)tasks.size();
-  a.tasks1 = (const BlockTask*)d_t1;
-  a.nblocks1 = (int)tasks1.size();
-  a.tasksu = (const BlockTask*)d_tu;
-  a.nblocksu = (int)tasksu.size();
-  a.ptasks = (const BlockTask*)d_pt;
-  a.npblocks = (int)ptasks.size();
   a.scratch = c->scratch;
   a.stepc = (char*)c->scratch + (size_t)stepc_off * es;
   a.gamma = c->prm.gamma;
@@ -763,11 +853,7 @@ static mhd_status advance_impl(mhd_ctx* c, const mhd_patch_desc* patches, int32_
   a.d_status = c->d_status;
   a.timer = timer_of(c);
   a.fused = fused;
-  a.items = (const FusedItem*)d_i;
-  a.nitems = (int)items.size();
   a.counter = (int*)((char*)c->scratch + counter_byte);
-  a.ctasks = (const BlockTask*)d_ct;
-  a.nctasks = (int)ctasks.size();
   a.variant = shape;
   a.commit = true;
   a.cfl_out = cfl_dt ? (unsigned long long*)const_cast<double*>(d_dt) : nullptr;
@@ -776,11 +862,6 @@ static mhd_status advance_impl(mhd_ctx* c, const mhd_patch_desc* patches, int32_
   a.rho_floor = c->prm.rho_floor;
   a.d_floors = c->d_floors;
   a.pf = pf;
-  if (pf) {
-    a.pf_items = (const FusedItem*)d_i;
-    a.npf = (int)items.size();
-    a.fused = false;
-  }
   cudaError_t e = run_advance_args(c, dtype, a, (cudaStream_t)stream);
   if (e != cudaSuccess) return cuda_fail(c, e, "patch advance launch");
   // fused: step constants, k_fused, k_commit; staged with the CFL dt: + reset
@@ -846,16 +927,12 @@ mhd_status mhd_autotune_advance(mhd_ctx* c, const mhd_patch_desc* patches, int32
   // after the work-queue head: a status word of the candidates' own, so that
   // their checks (on whatever the ghost zones hold) leave the context's alone
   if ((r = ensure_scratch(c, counter_byte + 32))) return r;
-  std::vector<BlockTask> tasks, tasks1, tasksu, ptasks;
-  staged_tasks(dp, elem_size(dtype), tasks, tasks1, tasksu);
-  pred_tiles(dp, dtype, ptasks);
-  if (tasks.size() > 0x7fffffff || ptasks.size() > 0x7fffffff) return fail(c, MHD_EINVAL, "launch too large");
-  void *d_p = nullptr, *d_t = nullptr, *d_t1 = nullptr, *d_tu = nullptr, *d_pt = nullptr;
+  const std::vector<PatchSize> ps = sizes_of(dp);
+  AdvanceArgs base{};
+  if ((r = staged_tables(c, ps, es, true, base))) return r;
+  if ((r = pred_table(c, dp, ps, dtype, base))) return r;
+  void* d_p = nullptr;
   if ((r = table(c, dp.data(), dp.size() * sizeof(DPatch), &d_p))) return r;
-  if ((r = table(c, tasks.data(), tasks.size() * sizeof(BlockTask), &d_t))) return r;
-  if ((r = table(c, tasks1.data(), tasks1.size() * sizeof(BlockTask), &d_t1))) return r;
-  if ((r = table(c, tasksu.data(), tasksu.size() * sizeof(BlockTask), &d_tu))) return r;
-  if ((r = table(c, ptasks.data(), ptasks.size() * sizeof(BlockTask), &d_pt))) return r;
   // the fused kernel's copy-back goes to planes of the scratch arena the
   // fused kernel does not use (the predicted-state planes), so that it is
   // timed without touching the patch state
@@ -906,21 +983,14 @@ mhd_status mhd_autotune_advance(mhd_ctx* c, const mhd_patch_desc* patches, int32
   float best = 3.4e38f;
   int bv = 0, bcz = 0;
   bool any = false;
-  std::vector<FusedItem> items;
-  std::vector<BlockTask> ctasks;
   int skip_shape = -1000;  // a shape this device cannot run: its other chunks are skipped
   for (const auto& cv : cand) {
     const int v = cv.first, cz = cv.second;
     if (v == skip_shape) continue;
-    AdvanceArgs a{};
+    AdvanceArgs a = base;
     a.patches = (const DPatch*)d_p;
     a.npatches = n;
-    a.tasks = (const BlockTask*)d_t;
-    a.nblocks = (int)tasks.size();
-    a.tasks1 = (const BlockTask*)d_t1;
-    a.nblocks1 = (int)tasks1.size();
-    a.tasksu = (const BlockTask*)d_tu;
-    a.nblocksu = (int)tasksu.size();
+    if (v != -1) a.npblocks = 0;  // the untiled predictor
     a.scratch = c->scratch;
     a.stepc = (char*)c->scratch + (size_t)stepc_off * es;
     a.gamma = c->prm.gamma;
@@ -935,41 +1005,21 @@ mhd_status mhd_autotune_advance(mhd_ctx* c, const mhd_patch_desc* patches, int32
     a.d_floors = c->d_floors;
     a.commit = false;  // every candidate leaves the patch state as it is
     a.fused = v >= 0;
-    if (v == -1) {
-      a.ptasks = (const BlockTask*)d_pt;
-      a.npblocks = (int)ptasks.size();
-    }
     if (v <= -3) {
-      const PfVariant& pv = dtype == MHD_F32 ? kPfVariants32[-3 - v] : kPfVariants64[-3 - v];
-      pf_items(dp, pv.tx, pv.ty, cz, items);
-      void* d_i = nullptr;
-      if ((r = table(c, items.data(), items.size() * sizeof(FusedItem), &d_i))) {
-        cudaEventDestroy(e0);
-        cudaEventDestroy(e1);
-        return r;
-      }
+      r = pf_table(c, dp, ps, dtype == MHD_F32 ? kPfVariants32[-3 - v] : kPfVariants64[-3 - v], cz, a);
       a.pf = true;
-      a.pf_items = (const FusedItem*)d_i;
-      a.npf = (int)items.size();
       a.variant = -3 - v;
     }
     if (a.fused) {
-      const FusedVariant& fv = fused_variant_of(dtype, v);
-      fused_items(dp, fv.bx, fv.by, cz, items, ctasks);
-      void *d_i = nullptr, *d_ct = nullptr;
-      if ((r = table(c, items.data(), items.size() * sizeof(FusedItem), &d_i)) ||
-          (r = table(c, ctasks.data(), ctasks.size() * sizeof(BlockTask), &d_ct))) {
-        cudaEventDestroy(e0);
-        cudaEventDestroy(e1);
-        return r;
-      }
-      a.items = (const FusedItem*)d_i;
-      a.nitems = (int)items.size();
+      r = fused_tables(c, dp, ps, fused_variant_of(dtype, v), cz, a);
       a.counter = (int*)((char*)c->scratch + counter_byte);
-      a.ctasks = (const BlockTask*)d_ct;
-      a.nctasks = (int)ctasks.size();
       a.variant = v;
       a.commit_patches = (const DPatch*)d_pc;
+    }
+    if (r) {
+      cudaEventDestroy(e0);
+      cudaEventDestroy(e1);
+      return r;
     }
     e = run_advance_args(c, dtype, a, s);
     if (e != cudaSuccess) {  // a shape this device cannot run: skip it
@@ -1028,16 +1078,16 @@ mhd_status mhd_cfl_dt(mhd_ctx* c, const mhd_patch_desc* patches, int32_t n, cons
     dp[p].cfl_scale = scale ? scale[p] : 1.0;
     counts[p] = (int64_t)dp[p].n[0] * dp[p].n[1] * dp[p].n[2];
   }
-  std::vector<BlockTask> tasks;
-  tasks_for(counts, tasks);
-  void *d_p = nullptr, *d_t = nullptr;
+  const BlockTask* d_t = nullptr;
+  int nblocks = 0;
+  if ((r = tasks_table(c, counts, &d_t, &nblocks))) return r;
+  void *d_p = nullptr;
   if ((r = table(c, dp.data(), dp.size() * sizeof(DPatch), &d_p))) return r;
-  if ((r = table(c, tasks.data(), tasks.size() * sizeof(BlockTask), &d_t))) return r;
-  cudaError_t e = cfl_dt_launch(dtype, (const DPatch*)d_p, (const BlockTask*)d_t, (int)tasks.size(),
+  cudaError_t e = cfl_dt_launch(dtype, (const DPatch*)d_p, d_t, nblocks,
                                 c->prm.gamma, c->prm.cfl, d_dt_out, c->d_status, timer_of(c),
                                 (cudaStream_t)stream);
   if (e != cudaSuccess) return cuda_fail(c, e, "cfl_dt launch");
-  c->launches += tasks.empty() ? 1 : 2;
+  c->launches += nblocks == 0 ? 1 : 2;
   return MHD_OK;
 }
 
@@ -1082,15 +1132,15 @@ mhd_status mhd_transfer_copy(mhd_ctx* c, const mhd_patch_desc* old, int32_t no, 
     }
     counts[t] = cnt;
   }
-  std::vector<BlockTask> tasks;
-  tasks_for(counts, tasks);
-  void *d_o = nullptr, *d_n = nullptr, *d_i = nullptr, *d_t = nullptr;
+  const BlockTask* d_t = nullptr;
+  int nblocks = 0;
+  if ((r = tasks_table(c, counts, &d_t, &nblocks))) return r;
+  void *d_o = nullptr, *d_n = nullptr, *d_i = nullptr;
   if ((r = table(c, dold.data(), dold.size() * sizeof(DPatch), &d_o))) return r;
   if ((r = table(c, dnew.data(), dnew.size() * sizeof(DPatch), &d_n))) return r;
   if ((r = table(c, it.data(), it.size() * sizeof(DTransfer), &d_i))) return r;
-  if ((r = table(c, tasks.data(), tasks.size() * sizeof(BlockTask), &d_t))) return r;
   cudaError_t e = transfer_copy_launch(dtype, (const DPatch*)d_o, (const DPatch*)d_n, (const DTransfer*)d_i,
-                                       (const BlockTask*)d_t, (int)tasks.size(), (cudaStream_t)stream);
+                                       d_t, nblocks, (cudaStream_t)stream);
   if (e != cudaSuccess) return cuda_fail(c, e, "transfer_copy launch");
   c->launches += 1;
   return MHD_OK;
@@ -1151,15 +1201,15 @@ mhd_status mhd_prolong_new(mhd_ctx* c, const mhd_patch_desc* coarse, int32_t nc,
     }
     nfall = c->d_counter;
   }
-  std::vector<BlockTask> tasks;
-  tasks_for(counts, tasks);
-  void *d_c = nullptr, *d_f = nullptr, *d_i = nullptr, *d_t = nullptr;
+  const BlockTask* d_t = nullptr;
+  int nblocks = 0;
+  if ((r = tasks_table(c, counts, &d_t, &nblocks))) return r;
+  void *d_c = nullptr, *d_f = nullptr, *d_i = nullptr;
   if ((r = table(c, dc.data(), dc.size() * sizeof(DPatch), &d_c))) return r;
   if ((r = table(c, df.data(), df.size() * sizeof(DPatch), &d_f))) return r;
   if ((r = table(c, it.data(), it.size() * sizeof(DProlongNew), &d_i))) return r;
-  if ((r = table(c, tasks.data(), tasks.size() * sizeof(BlockTask), &d_t))) return r;
   cudaError_t e = prolong_new_launch(dtype, (const DPatch*)d_c, (const DPatch*)d_f, (const DProlongNew*)d_i,
-                                     (const BlockTask*)d_t, (int)tasks.size(), energy_mode, nfall,
+                                     d_t, nblocks, energy_mode, nfall,
                                      (cudaStream_t)stream);
   if (e != cudaSuccess) return cuda_fail(c, e, "prolong_new launch");
   c->launches += 1;
@@ -1180,16 +1230,16 @@ mhd_status mhd_floor(mhd_ctx* c, const mhd_patch_desc* patches, int32_t n, void*
     dp[p].k = 0;
     counts[p] = (int64_t)(dp[p].n[0] + 1) * (dp[p].n[1] + 1) * (dp[p].n[2] + 1);
   }
-  std::vector<BlockTask> tasks;
-  tasks_for(counts, tasks);
-  void *d_p = nullptr, *d_t = nullptr;
+  const BlockTask* d_t = nullptr;
+  int nblocks = 0;
+  if ((r = tasks_table(c, counts, &d_t, &nblocks))) return r;
+  void *d_p = nullptr;
   if ((r = table(c, dp.data(), dp.size() * sizeof(DPatch), &d_p))) return r;
-  if ((r = table(c, tasks.data(), tasks.size() * sizeof(BlockTask), &d_t))) return r;
   AdvanceArgs a{};
   a.patches = (const DPatch*)d_p;
   a.npatches = n;
-  a.tasksu = (const BlockTask*)d_t;
-  a.nblocksu = (int)tasks.size();
+  a.tasksu = d_t;
+  a.nblocksu = nblocks;
   a.gamma = c->prm.gamma;
   a.p_floor = c->prm.p_floor;
   a.rho_floor = c->prm.rho_floor;
@@ -1231,67 +1281,31 @@ mhd_status mhd_flag_cells(mhd_ctx* c, const mhd_patch_desc* patches, int32_t n, 
     off[p] = total;
     total += counts[p];
   }
-  std::vector<BlockTask> tasks;
-  tasks_for(counts, tasks);
-  void *d_p = nullptr, *d_t = nullptr, *d_o = nullptr;
+  const BlockTask* d_t = nullptr;
+  int nblocks = 0;
+  if ((r = tasks_table(c, counts, &d_t, &nblocks))) return r;
+  void *d_p = nullptr, *d_o = nullptr;
   if ((r = table(c, dp.data(), dp.size() * sizeof(DPatch), &d_p))) return r;
-  if ((r = table(c, tasks.data(), tasks.size() * sizeof(BlockTask), &d_t))) return r;
   if ((r = table(c, off.data(), off.size() * sizeof(int64_t), &d_o))) return r;
-  cudaError_t e = flag_launch(dtype, (const DPatch*)d_p, (const BlockTask*)d_t, (int)tasks.size(),
+  cudaError_t e = flag_launch(dtype, (const DPatch*)d_p, d_t, nblocks,
                               (const int64_t*)d_o, c->prm.gamma, theta, d_flags, (cudaStream_t)stream);
   if (e != cudaSuccess) return cuda_fail(c, e, "flag_cells launch");
   c->launches += 1;
   return MHD_OK;
 }
 
-mhd_status mhd_ghost_fill(mhd_ctx* c, const mhd_patch_desc* patches, int32_t n, const mhd_copy* list,
-                          int32_t nlist, void* stream) {
-  mhd_status r = begin(c);
-  if (r) return r;
-  if (n < 0 || (n > 0 && !patches) || nlist < 0 || (nlist > 0 && !list))
-    return fail(c, MHD_EINVAL, "bad arguments");
-  if (nlist == 0) return MHD_OK;
-  std::vector<DPatch> dp(n);
-  const int dtype = n > 0 ? patches[0].dtype : 0;
-  for (int p = 0; p < n; ++p) {
-    if ((r = convert(c, patches[p], p, dp[p]))) return r;
-    if (patches[p].dtype != dtype) return fail(c, MHD_EINVAL, "patches of one call must share a dtype");
-  }
-  std::vector<DCopy> dc(nlist);
-  std::vector<int64_t> counts(nlist);
-  for (int t = 0; t < nlist; ++t) {
-    const mhd_copy& m = list[t];
-    if (m.src < 0 || m.src >= n || m.dst < 0 || m.dst >= n)
-      return fail(c, MHD_EINVAL, "copy %d: patch index out of range", t);
-    const DPatch& D = dp[m.dst];
-    const DPatch& S = dp[m.src];
-    DCopy& o = dc[t];
-    o.src = m.src;
-    o.dst = m.dst;
-    int64_t cnt = 1;
-    for (int a = 0; a < 3; ++a) {
-      const int lo = m.box.lo[a] - D.glo[a], hi = m.box.hi[a] - D.glo[a];
-      if (hi < lo || lo < -1 || hi > D.N[a])
-        return fail(c, MHD_EINVAL, "copy %d: box outside the destination's arrays grown by one along axis %d", t, a);
-      // source cells (and the upper face of the last one) must lie in src's interior
-      const int slo = m.box.lo[a] + m.offset[a] - S.glo[a], shi = m.box.hi[a] + m.offset[a] - S.glo[a];
-      if (slo < S.g || shi > S.g + S.n[a] - 1)
-        return fail(c, MHD_EINVAL, "copy %d: source outside the source interior along axis %d", t, a);
-      o.lo[a] = lo;
-      o.ext[a] = hi - lo + 1;
-      o.off[a] = (m.box.lo[a] + m.offset[a] - S.glo[a]) - lo;
-      cnt *= o.ext[a];
-    }
-    counts[t] = cnt;
-  }
-  // Bottom-layer rectangles: where copy u's top layer along a lies directly
-  // below copy t's bottom layer (same destination), the faces between them
-  // take u's values and t skips them over the transverse extent they share.
-  std::vector<std::vector<int32_t>> by_dst(n);
+// Bottom-layer rectangles of a fill's copies: where copy u's top layer along a
+// lies directly below copy t's bottom layer (same destination), the faces
+// between them take u's values and t skips them over the transverse extent
+// they share.
+static void ghost_rectangles(const std::vector<DCopy>& dc, int npatch, std::vector<DCopy>& out,
+                             std::vector<DExcl>& ex) {
+  const int nlist = (int)dc.size();
+  out = dc;
+  std::vector<std::vector<int32_t>> by_dst(npatch);
   for (int t = 0; t < nlist; ++t) by_dst[dc[t].dst].push_back(t);
-  std::vector<DExcl> ex;
   for (int t = 0; t < nlist; ++t) {
-    DCopy& o = dc[t];
+    DCopy& o = out[t];
     o.xr = (int32_t)ex.size();
     for (int32_t u : by_dst[o.dst]) {
       if (u == t) continue;
@@ -1314,25 +1328,84 @@ mhd_status mhd_ghost_fill(mhd_ctx* c, const mhd_patch_desc* patches, int32_t n, 
     o.nx = (int32_t)ex.size() - o.xr;
   }
   if (ex.empty()) ex.push_back(DExcl{});  // a valid table address
-  // warp tasks: groups of rows of each copy (lanes along x, see GhostTask)
-  std::vector<GhostTask> tasks;
+}
+
+// Warp tasks of a fill: groups of rows of each copy (lanes along x, see
+// GhostTask).
+static void ghost_tasks(const std::vector<DCopy>& dc, int dtype, std::vector<GhostTask>& tasks) {
   const int gr = ghost_rows(dtype);
-  for (int t = 0; t < nlist; ++t) {
+  for (size_t t = 0; t < dc.size(); ++t) {
     const DCopy& o = dc[t];
-    if ((int64_t)o.ext[1] * o.ext[2] >= (1 << 24))
-      return fail(c, MHD_EINVAL, "copy %d: more than 2^24 - 1 rows in one box", t);
     const int W = std::min(o.ext[0], 32), rows = o.ext[1] * o.ext[2], step = gr * (32 / W);
     for (int x0 = 0; x0 < o.ext[0]; x0 += 32)
-      for (int r0 = 0; r0 < rows; r0 += step) tasks.push_back(GhostTask{t, r0, x0, 0});
+      for (int r0 = 0; r0 < rows; r0 += step) tasks.push_back(GhostTask{(int32_t)t, r0, x0, 0});
   }
-  if (tasks.size() > 0x7fffffff / kThreads) return fail(c, MHD_EINVAL, "launch too large");
-  void *d_p = nullptr, *d_c = nullptr, *d_x = nullptr, *d_t = nullptr;
+}
+
+mhd_status mhd_ghost_fill(mhd_ctx* c, const mhd_patch_desc* patches, int32_t n, const mhd_copy* list,
+                          int32_t nlist, void* stream) {
+  mhd_status r = begin(c);
+  if (r) return r;
+  if (n < 0 || (n > 0 && !patches) || nlist < 0 || (nlist > 0 && !list))
+    return fail(c, MHD_EINVAL, "bad arguments");
+  if (nlist == 0) return MHD_OK;
+  std::vector<DPatch> dp(n);
+  const int dtype = n > 0 ? patches[0].dtype : 0;
+  for (int p = 0; p < n; ++p) {
+    if ((r = convert(c, patches[p], p, dp[p]))) return r;
+    if (patches[p].dtype != dtype) return fail(c, MHD_EINVAL, "patches of one call must share a dtype");
+  }
+  std::vector<DCopy> dc(nlist);
+  for (int t = 0; t < nlist; ++t) {
+    const mhd_copy& m = list[t];
+    if (m.src < 0 || m.src >= n || m.dst < 0 || m.dst >= n)
+      return fail(c, MHD_EINVAL, "copy %d: patch index out of range", t);
+    const DPatch& D = dp[m.dst];
+    const DPatch& S = dp[m.src];
+    DCopy& o = dc[t];
+    o.src = m.src;
+    o.dst = m.dst;
+    for (int a = 0; a < 3; ++a) {
+      const int lo = m.box.lo[a] - D.glo[a], hi = m.box.hi[a] - D.glo[a];
+      if (hi < lo || lo < -1 || hi > D.N[a])
+        return fail(c, MHD_EINVAL, "copy %d: box outside the destination's arrays grown by one along axis %d", t, a);
+      // source cells (and the upper face of the last one) must lie in src's interior
+      const int slo = m.box.lo[a] + m.offset[a] - S.glo[a], shi = m.box.hi[a] + m.offset[a] - S.glo[a];
+      if (slo < S.g || shi > S.g + S.n[a] - 1)
+        return fail(c, MHD_EINVAL, "copy %d: source outside the source interior along axis %d", t, a);
+      o.lo[a] = lo;
+      o.ext[a] = hi - lo + 1;
+      o.off[a] = (m.box.lo[a] + m.offset[a] - S.glo[a]) - lo;
+    }
+    if ((int64_t)o.ext[1] * o.ext[2] >= (1 << 24))
+      return fail(c, MHD_EINVAL, "copy %d: more than 2^24 - 1 rows in one box", t);
+  }
+  // The device tables: the copies with their bottom-layer rectangles, the
+  // rectangles, and the warp tasks, all functions of the resolved copies.
+  const size_t nkey = dc.size() * sizeof(DCopy);
+  std::vector<DCopy> full;
+  std::vector<DExcl> ex;
+  const DCopy* d_c = nullptr;
+  const DExcl* d_x = nullptr;
+  const GhostTask* d_t = nullptr;
+  int nc = 0, nx = 0, nt = 0;
+  auto rectangles = [&] {
+    if (full.empty()) ghost_rectangles(dc, n, full, ex);
+  };
+  r = keyed_table<DCopy>(
+      c, TK_GHOST_COPIES, dc.data(), nkey, [&](std::vector<DCopy>& v) { rectangles(), v = full; }, &d_c, &nc);
+  if (!r)
+    r = keyed_table<DExcl>(
+        c, TK_GHOST_EXCL, dc.data(), nkey, [&](std::vector<DExcl>& v) { rectangles(), v = ex; }, &d_x, &nx);
+  if (!r)
+    r = keyed_table<GhostTask>(
+        c, dtype == MHD_F32 ? TK_GHOST_TASKS32 : TK_GHOST_TASKS64, dc.data(), nkey,
+        [&](std::vector<GhostTask>& v) { ghost_tasks(dc, dtype, v); }, &d_t, &nt);
+  if (r) return r;
+  if (nt > 0x7fffffff / kThreads) return fail(c, MHD_EINVAL, "launch too large");
+  void* d_p = nullptr;
   if ((r = table(c, dp.data(), dp.size() * sizeof(DPatch), &d_p))) return r;
-  if ((r = table(c, dc.data(), dc.size() * sizeof(DCopy), &d_c))) return r;
-  if ((r = table(c, ex.data(), ex.size() * sizeof(DExcl), &d_x))) return r;
-  if ((r = table(c, tasks.data(), tasks.size() * sizeof(GhostTask), &d_t))) return r;
-  cudaError_t e = ghost_fill2_launch(dtype, (const DPatch*)d_p, (const DCopy*)d_c, (const DExcl*)d_x,
-                                     (const GhostTask*)d_t, (int)tasks.size(), timer_of(c), (cudaStream_t)stream);
+  cudaError_t e = ghost_fill2_launch(dtype, (const DPatch*)d_p, d_c, d_x, d_t, nt, timer_of(c), (cudaStream_t)stream);
   if (e != cudaSuccess) return cuda_fail(c, e, "ghost fill launch");
   c->launches += 1;
   return MHD_OK;
@@ -1351,13 +1424,13 @@ mhd_status mhd_conservation_sums(mhd_ctx* c, const mhd_patch_desc* patches, int3
     if (patches[p].dtype != dtype) return fail(c, MHD_EINVAL, "patches of one call must share a dtype");
     counts[p] = (int64_t)dp[p].n[0] * dp[p].n[1] * dp[p].n[2];
   }
-  std::vector<BlockTask> tasks;
-  tasks_for(counts, tasks);
-  if ((r = ensure_partials(c, tasks.size()))) return r;
-  void *d_p = nullptr, *d_t = nullptr;
+  const BlockTask* d_t = nullptr;
+  int nblocks = 0;
+  if ((r = tasks_table(c, counts, &d_t, &nblocks))) return r;
+  if ((r = ensure_partials(c, (size_t)nblocks))) return r;
+  void *d_p = nullptr;
   if ((r = table(c, dp.data(), dp.size() * sizeof(DPatch), &d_p))) return r;
-  if ((r = table(c, tasks.data(), tasks.size() * sizeof(BlockTask), &d_t))) return r;
-  cudaError_t e = sums_launch(dtype, (const DPatch*)d_p, (const BlockTask*)d_t, (int)tasks.size(),
+  cudaError_t e = sums_launch(dtype, (const DPatch*)d_p, d_t, nblocks,
                               c->partials, d_out8, timer_of(c), (cudaStream_t)stream);
   if (e != cudaSuccess) return cuda_fail(c, e, "sums launch");
   c->launches += 2;
@@ -1576,21 +1649,21 @@ mhd_status mhd_reflux(mhd_ctx* c, const mhd_patch_desc* coarse, int32_t nc, doub
     // elements one deposit element can flag: 2 for a face, 4 for an edge
     marks += cnt * (m.kind == 0 ? 2 : 4);
   }
-  std::vector<BlockTask> td;
-  tasks_for(dcount, td);
+  const BlockTask* d_td = nullptr;
+  int ntd = 0;
+  if ((r = tasks_table(c, dcount, &d_td, &ntd))) return r;
   // the list of flagged elements (and its count) in the arena
   if ((r = ensure_scratch(c, (size_t)(marks + 1) * 8))) return r;
   RefluxList L;
   L.count = (unsigned long long*)c->scratch;
   L.entries = L.count + 1;
   L.capacity = (unsigned long long)marks;
-  void *d_c = nullptr, *d_r = nullptr, *d_d = nullptr, *d_td = nullptr;
+  void *d_c = nullptr, *d_r = nullptr, *d_d = nullptr;
   if ((r = table(c, dc.data(), dc.size() * sizeof(DPatch), &d_c))) return r;
   if ((r = table(c, cr.data(), cr.size() * sizeof(DCorr), &d_r))) return r;
   if ((r = table(c, dd.data(), dd.size() * sizeof(DDeposit), &d_d))) return r;
-  if ((r = table(c, td.data(), td.size() * sizeof(BlockTask), &d_td))) return r;
   cudaError_t e = reflux_launch(dtype, (const DPatch*)d_c, (const DCorr*)d_r, L, (const DDeposit*)d_d,
-                                (const BlockTask*)d_td, (int)td.size(), timer_of(c), (cudaStream_t)stream);
+                                d_td, ntd, timer_of(c), (cudaStream_t)stream);
   if (e != cudaSuccess) return cuda_fail(c, e, "reflux launch");
   if (nd > 0) c->launches += 3;
   return MHD_OK;

@@ -9,12 +9,19 @@ PyTorch only provides the memory; every operation on it runs in
 """
 from __future__ import annotations
 
+import ctypes
 import itertools
+import struct
 from dataclasses import dataclass
 
 import torch
 
 from . import capi
+
+# mhd_patch_desc (include/mhd_gpu.h): level, nghost, dtype, patch_id, interior
+# lo and hi, U[5] and B[3], stride[3], dx[3]
+_DESC = struct.Struct("=10i8Q3q3d")
+assert _DESC.size == ctypes.sizeof(capi.mhd_patch_desc)
 
 DTYPES = {"f64": (torch.float64, capi.MHD_F64), "f32": (torch.float32, capi.MHD_F32)}
 
@@ -52,22 +59,12 @@ class Patch:
         st = self.state
         if not st.is_cuda or not st.is_contiguous():
             raise ValueError("patch state must be a contiguous CUDA tensor")
-        d = capi.mhd_patch_desc()
-        d.level = self.level
-        d.nghost = self.g
-        d.dtype = self.dtype_code
-        d.patch_id = self.patch_id
-        d.interior.lo[:] = tuple(int(v) for v in self.lo)
-        d.interior.hi[:] = tuple(int(v) for v in self.hi)
-        base = st.data_ptr()
-        plane = st.stride(0) * st.element_size()
-        for q in range(5):
-            d.U[q] = base + q * plane
-        for a in range(3):
-            d.B[a] = base + (5 + a) * plane
-        d.stride[:] = (1, st.stride(2), st.stride(1))
-        d.dx[:] = tuple(float(v) for v in self.dx)
-        return d
+        sq, sz, sy, _ = st.stride()
+        base, plane = st.data_ptr(), sq * st.element_size()
+        # the fields in the order of mhd_patch_desc, packed in one call
+        return capi.mhd_patch_desc.from_buffer_copy(_DESC.pack(
+            self.level, self.g, self.dtype_code, self.patch_id, *map(int, self.lo), *map(int, self.hi),
+            *range(base, base + 8 * plane, plane), 1, sy, sz, *map(float, self.dx)))
 
     @staticmethod
     def from_array(arr, lo, n, g, dx, dtype="f64", device="cuda", level=0, patch_id=0) -> "Patch":

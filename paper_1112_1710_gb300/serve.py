@@ -264,9 +264,7 @@ class GpuBackend:
         with torch.cuda.stream(s):
             for i, r in enumerate(batch):
                 tpl, dt = self.templates[(r.n, r.dtype)]
-                st = torch.empty_like(tpl.state)
-                st.copy_(tpl.state, non_blocking=True)
-                p = Patch(st, tpl.lo, tpl.n, tpl.g, tpl.dx, r.level, r.rid)
+                p = Patch(tpl.state.clone(), tpl.lo, tpl.n, tpl.g, tpl.dx, r.level, r.rid)
                 patches.append(p)
                 descs.append(p.desc())
                 scales.append(dt)
