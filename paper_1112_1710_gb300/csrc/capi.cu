@@ -43,6 +43,7 @@ enum TableKind : int {
   TK_PF_ITEMS,        // patch sizes, tile and chunk -> fused pass items
   TK_FUSED_ITEMS, TK_FUSED_TASKS,      // the same for the fused kernel
   TK_PACKED, TK_STARTS,                // element counts -> packed blocks, first elements
+  TK_FLAG_TILES,      // patch sizes -> tiles of the flag kernel
   TK_GHOST_COPIES, TK_GHOST_EXCL, TK_GHOST_TASKS64, TK_GHOST_TASKS32  // copies -> the ghost fill's tables
 };
 
@@ -235,6 +236,7 @@ mhd_status convert(mhd_ctx* c, const mhd_patch_desc& d, int idx, DPatch& o) {
     o.dxf[a] = (float)d.dx[a];
     o.rdx[a] = 1.0 / d.dx[a];
   }
+  o.dv = d.dx[0] * d.dx[1] * d.dx[2];
   if (d.stride[1] < N[0] + 1 || d.stride[2] < d.stride[1] * (N[1] + 1))
     return fail(c, MHD_EINVAL, "patch %d (id %d): strides too small for the face arrays", idx, d.patch_id);
   if (N[0] * N[1] * N[2] > (int64_t)1 << 31)
@@ -1264,26 +1266,53 @@ mhd_status mhd_floor_count(mhd_ctx* c, int64_t* out) {
   return MHD_OK;
 }
 
+// Tiles of the flag kernel: the interior's x extent in equal parts of at most 30
+// cells (a row of 32 threads with the rim), the y extent in equal parts of
+// what then fits the block, in chunks of planes.
+static void flag_tiles(const std::vector<PatchSize>& ps, std::vector<FusedItem>& out) {
+  for (size_t p = 0; p < ps.size(); ++p) {
+    const int32_t* n = ps[p].n;
+    const int nx = (n[0] + 29) / 30, tx = (n[0] + nx - 1) / nx;
+    const int ymax = kFlagThreads / (tx + 2) - 2, ny = (n[1] + ymax - 1) / ymax, ty = (n[1] + ny - 1) / ny;
+    for (int z0 = 0; z0 < n[2]; z0 += kFlagPlanes)
+      for (int y0 = 0; y0 < n[1]; y0 += ty)
+        for (int x0 = 0; x0 < n[0]; x0 += tx) {
+          FusedItem it{};
+          it.patch = (int32_t)p;
+          it.x0 = x0;
+          it.y0 = y0;
+          it.z0 = z0;
+          it.z1 = std::min(z0 + kFlagPlanes, (int)n[2]);
+          it.tx = std::min(tx, (int)n[0] - x0);
+          it.ty = std::min(ty, (int)n[1] - y0);
+          out.push_back(it);
+        }
+  }
+}
+
 mhd_status mhd_flag_cells(mhd_ctx* c, const mhd_patch_desc* patches, int32_t n, double theta, uint8_t* d_flags,
                           void* stream) {
   mhd_status r = begin(c);
   if (r) return r;
   if (n < 1 || !patches || !d_flags || !(theta >= 0.0)) return fail(c, MHD_EINVAL, "flag_cells: bad arguments");
   std::vector<DPatch> dp(n);
-  std::vector<int64_t> counts(n), off(n);
+  std::vector<int64_t> off(n);
   const int dtype = patches[0].dtype;
   int64_t total = 0;
   for (int p = 0; p < n; ++p) {
     if ((r = convert(c, patches[p], p, dp[p]))) return r;
     if (patches[p].dtype != dtype) return fail(c, MHD_EINVAL, "patches of one call must share a dtype");
     if (patches[p].nghost < 1) return fail(c, MHD_EINVAL, "flag_cells: patch %d needs a ghost layer", p);
-    counts[p] = (int64_t)dp[p].n[0] * dp[p].n[1] * dp[p].n[2];
     off[p] = total;
-    total += counts[p];
+    total += (int64_t)dp[p].n[0] * dp[p].n[1] * dp[p].n[2];
   }
-  const BlockTask* d_t = nullptr;
+  const std::vector<PatchSize> ps = sizes_of(dp);
+  const FusedItem* d_t = nullptr;
   int nblocks = 0;
-  if ((r = tasks_table(c, counts, &d_t, &nblocks))) return r;
+  r = keyed_table<FusedItem>(
+      c, TK_FLAG_TILES, ps.data(), ps.size() * sizeof(PatchSize),
+      [&](std::vector<FusedItem>& v) { flag_tiles(ps, v); }, &d_t, &nblocks);
+  if (r) return r;
   void *d_p = nullptr, *d_o = nullptr;
   if ((r = table(c, dp.data(), dp.size() * sizeof(DPatch), &d_p))) return r;
   if ((r = table(c, off.data(), off.size() * sizeof(int64_t), &d_o))) return r;

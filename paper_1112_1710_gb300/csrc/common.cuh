@@ -30,6 +30,7 @@ struct DPatch {
   float dxf[3];      // dx rounded to FP32 (FP32 kernels read no doubles per thread)
   int32_t pad2;
   double rdx[3];     // 1 / dx (FP64): the FP32-state refluxing multiplies by it
+  double dv;         // cell volume, dx[0] dx[1] dx[2]
 };
 
 // Cell width along d in the arithmetic type of a kernel.

@@ -207,6 +207,19 @@ template <int K> MHD_HD double scale(double x) {
   return value(s | r);
 }
 
+// The double equal to x, in integers (a conversion instruction takes the FP64
+// pipe's time).
+MHD_HD double widen(float x) {
+  const uint32_t f = fbits(x), m = f & 0x7fffffu, e = (f >> 23) & 0xffu, sign = f & 0x80000000u;
+  if (e - 1u < 0xfeu) return value(((uint64_t)(sign | (((f & 0x7fffffffu) >> 3) + (896u << 20))) << 32) | (uint64_t)(f << 29));
+  if (e == 0xffu) return value(((uint64_t)(sign | 0x7ff00000u | (m >> 3)) << 32) | (uint64_t)(m << 29));
+  if (m == 0) return value((uint64_t)sign << 32);
+  int k = 0;  // subnormal: the leading bit to position 23
+  uint32_t n = m;
+  while (!(n & 0x800000u)) n <<= 1, ++k;
+  return value(((uint64_t)(sign | ((uint32_t)(897 - k) << 20) | ((n & 0x7fffffu) >> 3)) << 32) | (uint64_t)(n << 29));
+}
+
 // x > 0, x < 0, x >= 0 (all false for NaN)
 MHD_HD bool pos(double x) { return bits(x) - 1u < 0x7ff0000000000000ull; }
 MHD_HD bool neg(double x) { return bits(x) - 0x8000000000000001ull < 0x7ff0000000000000ull; }

@@ -110,9 +110,12 @@ cudaError_t cfl_dt_launch(int dtype, const DPatch* patches, const BlockTask* tas
 cudaError_t sums_launch(int dtype, const DPatch* patches, const BlockTask* tasks, int nblocks,
                         double* partials, double* d_out8, const KernelTimer* tm, cudaStream_t s);
 
-// Regridding's error flags of the interiors (tasks span interiors; flags of
-// patch p start at off[p]).
-cudaError_t flag_launch(int dtype, const DPatch* patches, const BlockTask* tasks, int nblocks, const int64_t* off,
+// Regridding's error flags of the interiors (tasks: tiles of tx x ty interior
+// cells from (x0, y0), (tx + 2) (ty + 2) <= kFlagThreads, and at most
+// kFlagPlanes planes [z0, z1), in interior indices; flags of patch p start at
+// off[p]).
+constexpr int kFlagThreads = 512, kFlagPlanes = 16;
+cudaError_t flag_launch(int dtype, const DPatch* patches, const FusedItem* tasks, int nblocks, const int64_t* off,
                         double gamma, double theta, uint8_t* flags, cudaStream_t s);
 
 }  // namespace mhd

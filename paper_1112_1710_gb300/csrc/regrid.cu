@@ -28,7 +28,7 @@ __device__ __forceinline__ void rho_p(const DPatch& p, int64_t x, double gm1, do
   u[5] = 0.5 * ((double)((const R*)p.B[0])[x] + (double)((const R*)p.B[0])[x + 1]);
   u[6] = 0.5 * ((double)((const R*)p.B[1])[x] + (double)((const R*)p.B[1])[x + p.s1]);
   u[7] = 0.5 * ((double)((const R*)p.B[2])[x] + (double)((const R*)p.B[2])[x + p.s2]);
-  const double ir = 1.0 / u[0];
+  const double ir = i64::div(1.0, u[0]);
   const double vx = u[1] * ir, vy = u[2] * ir, vz = u[3] * ir;
   const double ke = 0.5 * u[0] * (vx * vx + vy * vy + vz * vz);
   const double me = 0.5 * (u[5] * u[5] + u[6] * u[6] + u[7] * u[7]);
@@ -36,23 +36,14 @@ __device__ __forceinline__ void rho_p(const DPatch& p, int64_t x, double gm1, do
   pr = gm1 * (u[4] - ke - me);
 }
 
-// One thread per interior cell: flagged when, for q in {rho, p} and some
-// axis d, |q(+d) - q(-d)| > theta (|q(+d)| + 2 |q| + |q(-d)|).
+// The FP64 decision for the cell at element x: flagged when, for q in {rho, p}
+// and some axis d, |q(+d) - q(-d)| > theta (|q(+d)| + 2 |q| + |q(-d)|).
 template <typename R>
-__global__ void __launch_bounds__(kThreads) k_flag(const DPatch* __restrict__ P, const BlockTask* __restrict__ T,
-                                                   const int64_t* __restrict__ off, double gm1, double theta,
-                                                   uint8_t* flags) {
-  const BlockTask t = T[blockIdx.x];
-  const DPatch& p = P[t.patch];
-  const int e = t.start + threadIdx.x;
-  const int nc = p.n[0] * p.n[1] * p.n[2];
-  if (e >= nc) return;
-  const int i = e % p.n[0], j = (e / p.n[0]) % p.n[1], k = e / (p.n[0] * p.n[1]);
-  const int64_t x = (int64_t)(p.g + i) + (int64_t)(p.g + j) * p.s1 + (int64_t)(p.g + k) * p.s2;
+__device__ __forceinline__ int flag_exact(const DPatch& p, int64_t x, double gm1, double theta) {
   double r0, p0;
   rho_p<R>(p, x, gm1, r0, p0);
   int f = 0;
-#pragma unroll
+#pragma unroll 1
   for (int d = 0; d < 3; ++d) {
     const int64_t sd = d == 0 ? 1 : (d == 1 ? p.s1 : p.s2);
     double rm, pm, rp, pp;
@@ -67,7 +58,118 @@ __global__ void __launch_bounds__(kThreads) k_flag(const DPatch* __restrict__ P,
       if (num > theta * den) f = 1;
     }
   }
-  flags[off[t.patch] + e] = (uint8_t)f;
+  return f;
+}
+
+// An FP32 value of the flagged quantities of one cell: density r, pressure p
+// and a bound d on |p - p64|.  With eps = 2^-24, each FP32 operation within
+// eps of its result and (for an FP64 state) each input within eps, ke is
+// within 9 eps, me within 8 eps mb where mb = (sum of the squared means of
+// |B| of the two faces) / 2 >= me, and E, two subtractions, gamma - 1 and
+// their product add 7 eps of |E| + ke + mb at most: 16 eps gm1 (|E| + ke + mb),
+// taken as 24.  Outside [1e-30, 1e30] the bound is infinite.
+struct FlagCell {
+  float r, p, d;
+};
+template <typename R> __device__ __forceinline__ FlagCell flag_cell(const DPatch& p, int64_t x, float gm1) {
+  const float rho = (float)((const R*)p.U[0])[x], mx = (float)((const R*)p.U[1])[x], my = (float)((const R*)p.U[2])[x],
+              mz = (float)((const R*)p.U[3])[x], E = (float)((const R*)p.U[4])[x];
+  const float x0 = (float)((const R*)p.B[0])[x], x1 = (float)((const R*)p.B[0])[x + 1];
+  const float y0 = (float)((const R*)p.B[1])[x], y1 = (float)((const R*)p.B[1])[x + p.s1];
+  const float z0 = (float)((const R*)p.B[2])[x], z1 = (float)((const R*)p.B[2])[x + p.s2];
+  const float bx = 0.5f * (x0 + x1), by = 0.5f * (y0 + y1), bz = 0.5f * (z0 + z1);
+  const float ax = 0.5f * (fabsf(x0) + fabsf(x1)), ay = 0.5f * (fabsf(y0) + fabsf(y1)), az = 0.5f * (fabsf(z0) + fabsf(z1));
+  const float ke = 0.5f * (mx * mx + my * my + mz * mz) * (1.0f / rho);
+  const float me = 0.5f * (bx * bx + by * by + bz * bz), mb = 0.5f * (ax * ax + ay * ay + az * az);
+  const float S = fabsf(E) + fabsf(ke) + mb;
+  FlagCell c;
+  c.r = rho;
+  c.p = gm1 * (E - ke - me);
+  c.d = (S > 1e-30f && S < 1e30f && fabsf(rho) > 1e-30f && fabsf(rho) < 1e30f) ? 1.5e-6f * gm1 * S : 1.0f / 0.0f;
+  return c;
+}
+
+// Sign of |a - b| - theta (|a| + 2 |c| + |b|) for values known within da, db,
+// dc: 1 above, -1 below, 0 not settled.  The rounding of the FP32 expressions
+// is within 2 eps num + 7 eps theta den, taken as 1e-6 of their sum; theta's
+// own rounding is inside; 1e-37 covers subnormal values.
+__device__ __forceinline__ int flag_side(float a, float b, float c, float da, float db, float dc, float theta) {
+  const float num = fabsf(a - b), t = theta * (fabsf(a) + 2.0f * fabsf(c) + fabsf(b));
+  const float m = 1.01f * ((da + db) + theta * (da + 2.0f * dc + db)) + 1e-6f * (num + t) + 1e-37f;
+  return num > t + m ? 1 : (num < t - m ? -1 : 0);
+}
+
+// A block takes a tile of tx x ty interior cells (it.tx + 2) (it.ty + 2) <=
+// kFlagThreads, one thread per cell of the tile grown by one, and marches
+// over the tile's chunk of planes: each cell's density and pressure are
+// computed once per tile in FP32, with a bound on their error, the plane's in
+// shared memory, the planes below and above in registers.  The decision is
+// taken on them where the bound leaves no doubt; the other cells go to a list
+// and are decided at the end by the FP64 expressions, so the flags are those
+// of FP64.  (Seven FP64 pressures per cell took 230 FP64 instructions and
+// bound the kernel to the FP64 pipe.)  Measured on 200 patches of 8^3-64^3
+// cells (4.0 M cells, FP32): 2,300 -> 88 us; a first version with a fixed
+// tile, its rim computed by a third of the threads and the FP64 decision in
+// the loop took 138 us.
+template <typename R>
+__global__ void __launch_bounds__(kFlagThreads, 2) k_flag(const DPatch* __restrict__ P,
+                                                          const FusedItem* __restrict__ T,
+                                                          const int64_t* __restrict__ off, double gm1, double theta,
+                                                          uint8_t* flags) {
+  __shared__ float sr[2][kFlagThreads], sp[2][kFlagThreads], sd[2][kFlagThreads];
+  __shared__ uint16_t list[kFlagThreads * kFlagPlanes];
+  __shared__ int nlist;
+  const FusedItem t = T[blockIdx.x];
+  const DPatch& p = P[t.patch];
+  const int W = t.tx + 2, r = threadIdx.x;
+  int lx;
+  const int ly = divmod24(r, W, lx);
+  const bool act = ly < t.ty + 2;
+  const bool in = act && lx > 0 && lx <= t.tx && ly > 0 && ly <= t.ty;
+  const int i = t.x0 + lx - 1, j = t.y0 + ly - 1;   // interior indices, -1 .. n
+  const float gm1f = (float)gm1, thf = (float)theta;
+  const int64_t s2 = p.s2;
+  const int64_t col = (int64_t)(p.g + i) + (int64_t)(p.g + j) * p.s1 + (int64_t)p.g * s2;
+  uint8_t* out = flags + off[t.patch] + i + (int64_t)p.n[0] * j;
+  const int64_t plane = (int64_t)p.n[0] * p.n[1];
+  if (r == 0) nlist = 0;
+  FlagCell zm{}, z0{}, zp{};
+  if (in) zm = flag_cell<R>(p, col + (t.z0 - 1) * s2, gm1f);
+  if (act) z0 = flag_cell<R>(p, col + t.z0 * s2, gm1f);
+  for (int z = t.z0; z < t.z1; ++z) {
+    const int b = z & 1;
+    sr[b][r] = z0.r;
+    sp[b][r] = z0.p;
+    sd[b][r] = z0.d;
+    if (in || (act && z + 1 < t.z1)) zp = flag_cell<R>(p, col + (z + 1) * s2, gm1f);
+    __syncthreads();
+    if (in) {
+      int f = 0, open = 0;
+      auto test = [&](const FlagCell& lo, const FlagCell& hi) {
+        const float eps = 1.2e-7f;  // an FP64 state's density within 2^-24
+        const int a = flag_side(hi.r, lo.r, z0.r, eps * fabsf(hi.r), eps * fabsf(lo.r), eps * fabsf(z0.r), thf);
+        const int c = flag_side(hi.p, lo.p, z0.p, hi.d, lo.d, z0.d, thf);
+        if (a > 0 || c > 0) f = 1;
+        if (a == 0 || c == 0) open = 1;
+      };
+      auto at = [&](int s) { return FlagCell{sr[b][s], sp[b][s], sd[b][s]}; };
+      test(at(r - 1), at(r + 1));
+      test(at(r - W), at(r + W));
+      test(zm, zp);
+      if (!f && open) list[atomicAdd(&nlist, 1)] = (uint16_t)((z - t.z0) * kFlagThreads + r);
+      out[plane * z] = (uint8_t)f;
+    }
+    zm = z0;
+    z0 = zp;
+  }
+  __syncthreads();
+  for (int e = r; e < nlist; e += kFlagThreads) {
+    int cx;
+    const int cy = divmod24(list[e] % kFlagThreads, W, cx);
+    const int ci = t.x0 + cx - 1, cj = t.y0 + cy - 1, ck = t.z0 + list[e] / kFlagThreads;
+    const int64_t x = (int64_t)(p.g + ci) + (int64_t)(p.g + cj) * p.s1 + (int64_t)(p.g + ck) * s2;
+    if (flag_exact<R>(p, x, gm1, theta)) flags[off[t.patch] + ci + (int64_t)p.n[0] * cj + plane * ck] = 1;
+  }
 }
 
 __device__ __forceinline__ int64_t lin3r(const DPatch& p, int i, int j, int k) {
@@ -362,13 +464,13 @@ __global__ void __launch_bounds__(kThreads) k_prolong_new(const DPatch* __restri
 
 }  // namespace
 
-cudaError_t flag_launch(int dtype, const DPatch* patches, const BlockTask* tasks, int nblocks, const int64_t* off,
+cudaError_t flag_launch(int dtype, const DPatch* patches, const FusedItem* tasks, int nblocks, const int64_t* off,
                         double gamma, double theta, uint8_t* flags, cudaStream_t s) {
   if (nblocks == 0) return cudaSuccess;
   if (dtype == 0)
-    k_flag<double><<<nblocks, kThreads, 0, s>>>(patches, tasks, off, gamma - 1.0, theta, flags);
+    k_flag<double><<<nblocks, kFlagThreads, 0, s>>>(patches, tasks, off, gamma - 1.0, theta, flags);
   else
-    k_flag<float><<<nblocks, kThreads, 0, s>>>(patches, tasks, off, gamma - 1.0, theta, flags);
+    k_flag<float><<<nblocks, kFlagThreads, 0, s>>>(patches, tasks, off, gamma - 1.0, theta, flags);
   return cudaGetLastError();
 }
 
