@@ -61,6 +61,25 @@ template <typename R> constexpr int kMuT = region_mu_top(sizeof(R));
 // into scratch planes (FP64).
 template <typename R> constexpr bool kInlineEdges = sizeof(R) == 4;
 
+// Blocks of the predictor and the flux kernel: a task's kThreads elements in
+// one block, or, in small FP64 launches, in blocks of 64.  FP64 runs at the FP64
+// pipe's rate, so an SM that holds one block more than the others decides the
+// time of a small launch (199 blocks of 256 on 152 SMs, 2D Orszag-Tang 128^2:
+// k_pred 101 -> 78 us, k_flux 92 -> 72 us with 64 threads); in large launches
+// the smaller blocks cost more (their warps drift apart in code of 3,000
+// instructions: 90 x 75 x 66 cells, 1,880 blocks, 1.43 -> 1.57 ms per step),
+// so the line lies at four blocks per SM, where the last block per SM is a
+// quarter of the time at most.
+__device__ __forceinline__ BlockTask fine_task(const BlockTask* __restrict__ T) {
+  const int split = kThreads / blockDim.x;
+  BlockTask t = T[blockIdx.x / split];
+  t.start += (int)(blockIdx.x % split) * blockDim.x;
+  return t;
+}
+inline int fine_threads(size_t elem, int nblocks, int nsm) {
+  return elem == 8 && nblocks < 4 * nsm ? 64 : kThreads;
+}
+
 template <typename R> struct SolverConsts {
   R gamma, gm1, igm1, eps_up;
   int limiter, emf;
@@ -364,7 +383,7 @@ template <typename R> struct RegSlopes {
 };
 
 // 8-value sets of one cell parked in shared memory as rows of 16-byte vectors,
-// kThreads to a row, each thread its own column (set d: FP32 rows 2d and
+// a block's threads to a row, each thread its own column (set d: FP32 rows 2d and
 // 2d + 1, FP64 rows 4d to 4d + 3).
 // The stores and loads are volatile asm, so that the compiler neither
 // forwards the stored values in registers nor moves a load above its store;
@@ -388,7 +407,7 @@ template <typename R> struct SmemSets {
   static constexpr int W = 16 / (int)sizeof(R);  // values per vector
   uint32_t base;  // shared address of row 0, this thread's column
   __device__ __forceinline__ uint32_t row(int d, int k) const {
-    return base + (uint32_t)(d * (8 / W) + k) * kThreads * 16;
+    return base + (uint32_t)(d * (8 / W) + k) * blockDim.x * 16;
   }
   __device__ __forceinline__ void put(int d, const R (&v)[8]) const {
 #pragma unroll
@@ -520,7 +539,7 @@ __global__ void __launch_bounds__(kThreads, sizeof(R) == 4 ? MHD_PRED_MINB : 2) 
                                                    SolverConsts<R> sc, const R* __restrict__ K) {
   using S = SmemSets<R>;
   extern __shared__ __align__(16) unsigned char pred_smem[];
-  const BlockTask t = T[blockIdx.x];
+  const BlockTask t = fine_task(T);
   const DPatch& p = P[t.patch];
   Cell c;
   if (!region_cell<kM1<R>, kM1<R>>(p, t.start + threadIdx.x, c)) return;
@@ -605,9 +624,9 @@ __global__ void __launch_bounds__(kThreads, sizeof(R) == 4 ? MHD_PRED_MINB : 2) 
   }
 }
 
-// Dynamic shared memory of k_pred: FP32 the slopes of three axes, FP64 six
-// conserved face states.
-template <typename R> constexpr size_t kPredSmem = sizeof(R) * (sizeof(R) == 4 ? 24 : 48) * kThreads;
+// Dynamic shared memory of k_pred per thread: FP32 the slopes of three axes,
+// FP64 six conserved face states.
+template <typename R> constexpr size_t kPredSmem = sizeof(R) * (sizeof(R) == 4 ? 24 : 48);
 
 // Tiled predictor: a block owns a TX x TY x TZ tile of UB+1 cells (its task's
 // `start` is the tile index within the patch), stages W on the tile grown by
@@ -717,7 +736,7 @@ template <typename R>
 __global__ void __launch_bounds__(kThreads, sizeof(R) == 4 ? 4 : 2) k_flux(const DPatch* __restrict__ P,
                                                    const BlockTask* __restrict__ T, R* scr,
                                                    SolverConsts<R> sc, const R* __restrict__ K) {
-  const BlockTask t = T[blockIdx.x];
+  const BlockTask t = fine_task(T);
   const DPatch& p = P[t.patch];
   Cell c;
   if (!region_cell<kM1<R>, kM1<R>>(p, t.start + threadIdx.x, c)) return;
@@ -1069,7 +1088,8 @@ cudaError_t launch_advance(const AdvanceArgs& a, R* scr, R* K, const SolverConst
   const KernelTimer* tm = a.timer;
   const bool commit = a.commit;
   if (a.nblocks == 0) return cudaSuccess;
-  const dim3 g1(a.nblocks), g1b(a.nblocks1), gu(a.nblocksu);
+  const int bf = fine_threads(sizeof(R), a.nblocks1, a.nsm);
+  const dim3 g1(a.nblocks), g1f(a.nblocks1 * (kThreads / bf)), gu(a.nblocksu);
   if (a.cfl_out) {
     // the step's own CFL dt first (k_prim), then the step constants from it
     MHD_TIMED(tm, K_PRIM, s,
@@ -1086,13 +1106,13 @@ cudaError_t launch_advance(const AdvanceArgs& a, R* scr, R* K, const SolverConst
   else
     {
     static bool configured[64] = {};
-    const cudaError_t e = allow_smem(k_pred<R>, kPredSmem<R>, configured);
+    const cudaError_t e = allow_smem(k_pred<R>, kPredSmem<R> * kThreads, configured);
     if (e != cudaSuccess) return e;
-    MHD_TIMED(tm, K_PRED, s, (k_pred<R><<<g1b, kThreads, kPredSmem<R>, s>>>(d_patches, d_tasks1, scr, sc, K)));
+    MHD_TIMED(tm, K_PRED, s, (k_pred<R><<<g1f, bf, kPredSmem<R> * bf, s>>>(d_patches, d_tasks1, scr, sc, K)));
   }
   constexpr bool inl = kInlineEdges<R>;
   if (!inl) MHD_TIMED(tm, K_EDGE, s, (k_edge<R><<<g1, kThreads, 0, s>>>(d_patches, d_tasks, scr)));
-  MHD_TIMED(tm, K_FLUX, s, (k_flux<R><<<g1b, kThreads, 0, s>>>(d_patches, d_tasks1, scr, sc, K)));
+  MHD_TIMED(tm, K_FLUX, s, (k_flux<R><<<g1f, bf, 0, s>>>(d_patches, d_tasks1, scr, sc, K)));
   if (!inl) MHD_TIMED(tm, K_EMF, s, (k_emf<R><<<gu, kThreads, 0, s>>>(d_patches, d_tasksu, scr, sc)));
   MHD_TIMED(tm, K_UPDATE, s,
             (k_update<R, inl><<<gu, kThreads, 0, s>>>(d_patches, d_tasksu, scr, sc, K, commit ? 1 : 0)));

@@ -73,6 +73,7 @@ uint64_t hash_bytes(int kind, const void* p, size_t n) {
 struct mhd_ctx {
   mhd_params prm;
   int device = 0;
+  int nsm = 1;
   void* scratch = nullptr;
   size_t scratch_bytes = 0;
   double* partials = nullptr;
@@ -433,6 +434,7 @@ mhd_status mhd_ctx_create(const mhd_params* params, int32_t device, mhd_ctx** ou
   c->prm = *params;
   c->device = device;
   cudaError_t e = cudaSetDevice(device);
+  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&c->nsm, cudaDevAttrMultiProcessorCount, device);
   if (e == cudaSuccess) e = cudaMalloc(&c->d_status, sizeof(int));
   if (e == cudaSuccess) e = cudaMemset(c->d_status, 0, sizeof(int));
   if (e == cudaSuccess) e = cudaMalloc(&c->d_floors, sizeof(unsigned long long));
@@ -825,6 +827,7 @@ static mhd_status advance_impl(mhd_ctx* c, const mhd_patch_desc* patches, int32_
   if (shape >= (pf ? (di ? kNumPf32 : kNumPf64) : (di ? kNumFused32 : kNumFused64)))
     return fail(c, MHD_EINVAL, "kernel_shape %d is not compiled for this element type", c->prm.kernel_shape);
   AdvanceArgs a{};
+  a.nsm = c->nsm;
   const std::vector<PatchSize> ps = sizes_of(dp);
   if (pf) {
     const int cz = c->prm.fused_chunk > 0 ? c->prm.fused_chunk : c->fused_chunk[di] > 0 ? c->fused_chunk[di] : 16;
@@ -931,6 +934,7 @@ mhd_status mhd_autotune_advance(mhd_ctx* c, const mhd_patch_desc* patches, int32
   if ((r = ensure_scratch(c, counter_byte + 32))) return r;
   const std::vector<PatchSize> ps = sizes_of(dp);
   AdvanceArgs base{};
+  base.nsm = c->nsm;
   if ((r = staged_tables(c, ps, es, true, base))) return r;
   if ((r = pred_table(c, dp, ps, dtype, base))) return r;
   void* d_p = nullptr;

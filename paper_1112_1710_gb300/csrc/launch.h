@@ -10,6 +10,7 @@ namespace mhd {
 struct AdvanceArgs {
   const DPatch* patches;   // device
   int npatches;
+  int nsm;                 // the device's SM count
   const BlockTask* tasks;  // device, blocks over each patch's UB+2
   int nblocks;
   const BlockTask* tasks1;  // device, blocks over each patch's UB+1
