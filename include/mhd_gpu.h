@@ -95,8 +95,11 @@ typedef struct {
                         multiply-add; every operation rounded as written, in
                         the oracle's order), 1 the build with multiply-adds
                         fused (about 1.25x faster; differs from 0 by rounding) */
-  int32_t advance_kernel; /* 0: the context's choice (the staged kernels until
-                        mhd_autotune_advance measured something else faster);
+  int32_t advance_kernel; /* 0: the context's choice (what mhd_autotune_advance
+                        measured fastest; before that the fused pass for
+                        MHD_F32 calls without captures and grown boxes, in
+                        mhd_patch_step_cfl only if the patches fill the
+                        device, else the staged kernels);
                         1: the staged kernels (one launch per stage,
                         intermediates in the scratch arena; the predictor
                         tiled in shared memory if the autotuner chose it);
@@ -108,12 +111,13 @@ typedef struct {
                         Riemann fluxes over x-y tiles marching along z, the
                         predicted face states kept on chip), then the staged
                         EMF and update kernels.  All compute every element
-                        with the same expressions; a call whose captures need
+                        with the same expressions (in MHD_F32 the fused pass
+                        to rounding); a call whose captures need
                         face fluxes outside the update box runs staged (2) or
                         takes them from the fused pass's flux planes (4).   */
   int32_t fused_chunk; /* z-planes per work item of the fused kernel (2) or
                         of the fused pass (4); 0 lets each call choose (from
-                        the device's SM count for 2, 16 planes for 4)        */
+                        the device's SM count and the patch sizes)           */
   int32_t kernel_shape; /* compiled tile shape of the fused kernel (2) or of
                         the fused pass (4): 0 the context's choice (the first
                         shape until mhd_autotune_advance chose one); s >= 1

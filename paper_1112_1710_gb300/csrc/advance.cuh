@@ -70,7 +70,8 @@ template <typename R> constexpr bool kInlineEdges = sizeof(R) == 4;
 // instructions: 90 x 75 x 66 cells, 1,880 blocks, 1.43 -> 1.57 ms per step),
 // so the line lies at four blocks per SM, where the last block per SM is a
 // quarter of the time at most.
-__device__ __forceinline__ BlockTask fine_task(const BlockTask* __restrict__ T) {
+template <typename R> __device__ __forceinline__ BlockTask fine_task(const BlockTask* __restrict__ T) {
+  if constexpr (sizeof(R) == 4) return T[blockIdx.x];
   const int split = kThreads / blockDim.x;
   BlockTask t = T[blockIdx.x / split];
   t.start += (int)(blockIdx.x % split) * blockDim.x;
@@ -254,6 +255,56 @@ template <typename R> struct StepDt {
   }
 };
 
+// Primitives of the cell at element x from the state (no floors).
+template <typename R>
+__device__ __forceinline__ void load_prim(const DPatch& p, int64_t x, const SolverConsts<R>& sc, R (&w)[8]) {
+  R u[8];
+#pragma unroll
+  for (int q = 0; q < 5; ++q) u[q] = ((const R*)p.U[q])[x];
+  u[5] = Tr<R>::half(((const R*)p.B[0])[x] + ((const R*)p.B[0])[x + 1]);
+  u[6] = Tr<R>::half(((const R*)p.B[1])[x] + ((const R*)p.B[1])[x + p.s1]);
+  u[7] = Tr<R>::half(((const R*)p.B[2])[x] + ((const R*)p.B[2])[x + p.s2]);
+  cons2prim(u, sc.gm1, w);
+}
+
+// A cell's CFL candidate min_d dx_d / (|v_d| + c_f,d).
+template <typename R>
+__device__ __forceinline__ R cfl_candidate(const DPatch& p, const R (&w)[8], const SolverConsts<R>& sc) {
+  R m = R(1) / R(0);
+#pragma unroll
+  for (int d = 0; d < 3; ++d) {
+    const int t1 = (d + 1) % 3, t2 = (d + 2) % 3;
+    R cf = fast_speed(w[0], w[4], w[5 + d], w[5 + t1], w[5 + t2], sc.gamma);
+    R tt = Tr<R>::div(dx_of<R>(p, d), Tr<R>::abs(w[1 + d]) + cf);
+    m = rmin(m, tt);
+  }
+  return m;
+}
+
+// The block's smallest candidate lowers *dt_bits (every thread takes part).
+template <typename R>
+__device__ __forceinline__ void reduce_dt(R m, const DPatch& p, double cfl, unsigned long long* dt_bits) {
+  const R inf = R(1) / R(0);
+  for (int o = 16; o > 0; o >>= 1) {
+    R u2 = __shfl_down_sync(0xffffffffu, m, o);
+    m = (u2 < m) ? u2 : m;
+  }
+  __shared__ R red[kThreads / 32];
+  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = m;
+  __syncthreads();
+  if (threadIdx.x < 32) {
+    m = (threadIdx.x < kThreads / 32) ? red[threadIdx.x] : inf;
+    for (int o = 16; o > 0; o >>= 1) {
+      R u2 = __shfl_down_sync(0xffffffffu, m, o);
+      m = (u2 < m) ? u2 : m;
+    }
+    if (threadIdx.x == 0) {
+      const double v = (cfl * (double)m) * p.cfl_scale;
+      if (v == v) atomicMin(dt_bits, (unsigned long long)__double_as_longlong(v));
+    }
+  }
+}
+
 // ---------------------------------------------------------------- k_prim
 // Primitives and cell EMFs on UB+2.  With Cfl, also the CFL time step of the
 // step (the quantity mhd_cfl_dt computes, with the same expressions): each
@@ -276,27 +327,13 @@ __global__ void __launch_bounds__(kThreads) k_prim(const DPatch* __restrict__ P,
   R m = inf;
   if (act) {
     const int64_t x = lin(p, c);
-    R u[8];
-#pragma unroll
-    for (int q = 0; q < 5; ++q) u[q] = ((const R*)p.U[q])[x];
-    u[5] = Tr<R>::half(((const R*)p.B[0])[x] + ((const R*)p.B[0])[x + 1]);
-    u[6] = Tr<R>::half(((const R*)p.B[1])[x] + ((const R*)p.B[1])[x + p.s1]);
-    u[7] = Tr<R>::half(((const R*)p.B[2])[x] + ((const R*)p.B[2])[x + p.s2]);
     R w[8];
-    cons2prim(u, sc.gm1, w);
+    load_prim(p, x, sc, w);
     if constexpr (Cfl) {
       // the CFL candidate from the unfloored primitives (as mhd_cfl_dt)
       const bool interior = c.i >= p.g && c.i < p.g + p.n[0] && c.j >= p.g && c.j < p.g + p.n[1] &&
                             c.k >= p.g && c.k < p.g + p.n[2];
-      if (interior) {
-#pragma unroll
-        for (int d = 0; d < 3; ++d) {
-          const int t1 = (d + 1) % 3, t2 = (d + 2) % 3;
-          R cf = fast_speed(w[0], w[4], w[5 + d], w[5 + t1], w[5 + t2], sc.gamma);
-          R tt = Tr<R>::div(dx_of<R>(p, d), Tr<R>::abs(w[1 + d]) + cf);
-          m = rmin(m, tt);
-        }
-      }
+      if (interior) m = cfl_candidate(p, w, sc);
     }
     // the floors (when set) bound the primitives the step reads, ghost cells
     // included
@@ -310,26 +347,26 @@ __global__ void __launch_bounds__(kThreads) k_prim(const DPatch* __restrict__ P,
     }
     if (!Tr<R>::pos(w[0]) || !Tr<R>::pos(w[4])) raise_status(status, -4);
   }
-  if constexpr (Cfl) {
-    for (int o = 16; o > 0; o >>= 1) {
-      R u2 = __shfl_down_sync(0xffffffffu, m, o);
-      m = (u2 < m) ? u2 : m;
-    }
-    __shared__ R red[kThreads / 32];
-    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = m;
-    __syncthreads();
-    if (threadIdx.x < 32) {
-      m = (threadIdx.x < kThreads / 32) ? red[threadIdx.x] : inf;
-      for (int o = 16; o > 0; o >>= 1) {
-        R u2 = __shfl_down_sync(0xffffffffu, m, o);
-        m = (u2 < m) ? u2 : m;
-      }
-      if (threadIdx.x == 0) {
-        const double v = (cfl * (double)m) * p.cfl_scale;
-        if (v == v) atomicMin(dt_bits, (unsigned long long)__double_as_longlong(v));
-      }
-    }
+  if constexpr (Cfl) reduce_dt(m, p, cfl, dt_bits);
+}
+
+// The CFL time step alone, from the interiors of [lo, hi + 1] (k_prim's
+// expressions): the fused pass keeps its primitives on chip and needs the dt
+// before it starts.
+template <typename R>
+__global__ void __launch_bounds__(kThreads) k_cfl_step(const DPatch* __restrict__ P, const BlockTask* __restrict__ T,
+                                                       SolverConsts<R> sc, double cfl, unsigned long long* dt_bits) {
+  const BlockTask t = T[blockIdx.x];
+  const DPatch& p = P[t.patch];
+  Cell c;
+  R m = R(1) / R(0);
+  if (region_cell<kMu<R>, kMuT<R>>(p, t.start + threadIdx.x, c) && c.i < p.g + p.n[0] && c.j < p.g + p.n[1] &&
+      c.k < p.g + p.n[2]) {
+    R w[8];
+    load_prim(p, lin(p, c), sc, w);
+    m = cfl_candidate(p, w, sc);
   }
+  reduce_dt(m, p, cfl, dt_bits);
 }
 
 // Sets the FP64 time step the CFL reduction of k_prim lowers to +infinity.
@@ -407,7 +444,7 @@ template <typename R> struct SmemSets {
   static constexpr int W = 16 / (int)sizeof(R);  // values per vector
   uint32_t base;  // shared address of row 0, this thread's column
   __device__ __forceinline__ uint32_t row(int d, int k) const {
-    return base + (uint32_t)(d * (8 / W) + k) * blockDim.x * 16;
+    return base + (uint32_t)(d * (8 / W) + k) * (sizeof(R) == 4 ? (uint32_t)kThreads : blockDim.x) * 16;
   }
   __device__ __forceinline__ void put(int d, const R (&v)[8]) const {
 #pragma unroll
@@ -539,7 +576,7 @@ __global__ void __launch_bounds__(kThreads, sizeof(R) == 4 ? MHD_PRED_MINB : 2) 
                                                    SolverConsts<R> sc, const R* __restrict__ K) {
   using S = SmemSets<R>;
   extern __shared__ __align__(16) unsigned char pred_smem[];
-  const BlockTask t = fine_task(T);
+  const BlockTask t = fine_task<R>(T);
   const DPatch& p = P[t.patch];
   Cell c;
   if (!region_cell<kM1<R>, kM1<R>>(p, t.start + threadIdx.x, c)) return;
@@ -736,7 +773,7 @@ template <typename R>
 __global__ void __launch_bounds__(kThreads, sizeof(R) == 4 ? 4 : 2) k_flux(const DPatch* __restrict__ P,
                                                    const BlockTask* __restrict__ T, R* scr,
                                                    SolverConsts<R> sc, const R* __restrict__ K) {
-  const BlockTask t = fine_task(T);
+  const BlockTask t = fine_task<R>(T);
   const DPatch& p = P[t.patch];
   Cell c;
   if (!region_cell<kM1<R>, kM1<R>>(p, t.start + threadIdx.x, c)) return;
@@ -809,6 +846,32 @@ template <int a> __device__ __forceinline__ float emf_avg4(const DPatch& p, int6
   return 0.25f * (eb_lo + eb_hi + ec_lo + ec_hi);
 }
 
+// FP32 EMFs (emf_at's values) of the three edges stored at element x: the
+// induction fluxes and contact sides as the nine float4 vectors of slots 4-7
+// around the edges, instead of 24 scalars at a 16-byte stride.
+__device__ __forceinline__ void emf_up4(const DPatch& p, int64_t x, const float* scr, int emf, float (&e)[3]) {
+  const int64_t s[3] = {1, p.s1, p.s2};
+  float g[3][3][4];  // [axis][0 at x, 1 and 2 at x - the next axes' strides][slot - 4]
+#pragma unroll
+  for (int d = 0; d < 3; ++d) {
+    const float4* F = reinterpret_cast<const float4*>(arr(scr, p, SC_F + d * 8) + 4 * p.snelem);
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+      const float4 v = F[k == 0 ? x : x - s[(d + k) % 3]];
+      g[d][k][0] = v.x; g[d][k][1] = v.y; g[d][k][2] = v.z; g[d][k][3] = v.w;
+    }
+  }
+#pragma unroll
+  for (int a = 0; a < 3; ++a) {
+    const int b = (a + 1) % 3, c = (a + 2) % 3;
+    const float* Er = arr(scr, p, SC_ER + a);
+    // the b-faces at x and x - s_c, the c-faces at x and x - s_b
+    e[a] = edge_emf_value(-g[b][1][1 + c], -g[b][0][1 + c], g[c][2][1 + b], g[c][0][1 + b], Er[x - s[b] - s[c]],
+                          Er[x - s[c]], Er[x - s[b]], Er[x], g[b][1][1 + b], g[b][0][1 + b], g[c][2][1 + c],
+                          g[c][0][1 + c], emf);
+  }
+}
+
 // Is the axis-a edge stored at cell c one of the edges of the update box's
 // faces (the edges whose EMF the flux registers capture)?
 template <int a> __device__ __forceinline__ bool update_edge(const DPatch& p, const Cell& c) {
@@ -831,9 +894,15 @@ __global__ void __launch_bounds__(kThreads) k_emf(const DPatch* __restrict__ P,
   const R* cs = scr;
   const bool u0 = update_edge<0>(p, c), u1 = update_edge<1>(p, c), u2 = update_edge<2>(p, c);
   R e0 = R(0), e1 = R(0), e2 = R(0);
-  if (u0) e0 = emf_at<R, 0>(p, x, cs, sc.emf);
-  if (u1) e1 = emf_at<R, 1>(p, x, cs, sc.emf);
-  if (u2) e2 = emf_at<R, 2>(p, x, cs, sc.emf);
+  if constexpr (sizeof(R) == 4) {
+    R e[3];  // (the reads stay inside UB+1's planes)
+    emf_up4(p, x, cs, sc.emf, e);
+    e0 = e[0]; e1 = e[1]; e2 = e[2];
+  } else {
+    if (u0) e0 = emf_at<R, 0>(p, x, cs, sc.emf);
+    if (u1) e1 = emf_at<R, 1>(p, x, cs, sc.emf);
+    if (u2) e2 = emf_at<R, 2>(p, x, cs, sc.emf);
+  }
   if (u0) arr(scr, p, SC_ED + 0)[x] = e0;
   if (u1) arr(scr, p, SC_ED + 1)[x] = e1;
   if (u2) arr(scr, p, SC_ED + 2)[x] = e2;
@@ -1031,6 +1100,21 @@ template <typename F> cudaError_t allow_smem(F f, size_t smem, bool (&configured
   return e;
 }
 
+// Enqueues the edge EMFs and the update.
+template <typename R>
+void launch_update(const AdvanceArgs& a, R* scr, R* K, const SolverConsts<R>& sc, cudaStream_t s) {
+  const KernelTimer* tm = a.timer;
+  const int commit = a.commit ? 1 : 0;
+  if (update_emf_inline(sizeof(R), a.emf, a.nblocksu, a.nsm)) {
+    MHD_TIMED(tm, K_UPDATE, s,
+              (k_update<R, true><<<a.nblocksu, kThreads, 0, s>>>(a.patches, a.tasksu, scr, sc, K, commit)));
+  } else {
+    MHD_TIMED(tm, K_EMF, s, (k_emf<R><<<a.nblocksu, kThreads, 0, s>>>(a.patches, a.tasksu, scr, sc)));
+    MHD_TIMED(tm, K_UPDATE, s,
+              (k_update<R, false><<<a.nblocksu, kThreads, 0, s>>>(a.patches, a.tasksu, scr, sc, K, commit)));
+  }
+}
+
 // Enqueues the step constants, the fused pass of compiled shape TX x TY and
 // the staged EMF / update / floor kernels.
 template <typename R, int TX, int TY, int MINB>
@@ -1042,14 +1126,15 @@ cudaError_t launch_pf_shape(const AdvanceArgs& a, R* scr, R* K, const SolverCons
   const cudaError_t e = allow_smem(k_pf<R, TX, TY, MINB>, smem, configured);
   if (e != cudaSuccess) return e;
   const KernelTimer* tm = a.timer;
+  if (a.cfl_out)
+    MHD_TIMED(tm, K_CFL, s,
+              (k_dt_reset<<<1, 1, 0, s>>>(a.cfl_out),
+               k_cfl_step<R><<<a.nblocksu, kThreads, 0, s>>>(a.patches, a.tasksu, sc, a.cfl, a.cfl_out)));
   MHD_TIMED(tm, K_PF, s,
             (k_stepc<R><<<(a.npatches + 127) / 128, 128, 0, s>>>(a.patches, a.npatches, a.d_dt, K),
              k_pf<R, TX, TY, MINB><<<a.npf, L::NT, smem, s>>>(a.patches, a.pf_items, scr, K, sc, a.d_status)));
-  constexpr bool inl = kInlineEdges<R>;
+  launch_update<R>(a, scr, K, sc, s);
   const dim3 gu(a.nblocksu);
-  if (!inl) MHD_TIMED(tm, K_EMF, s, (k_emf<R><<<gu, kThreads, 0, s>>>(a.patches, a.tasksu, scr, sc)));
-  MHD_TIMED(tm, K_UPDATE, s,
-            (k_update<R, inl><<<gu, kThreads, 0, s>>>(a.patches, a.tasksu, scr, sc, K, a.commit ? 1 : 0)));
   if (a.commit && (a.p_floor > 0.0 || a.rho_floor > 0.0))
     MHD_TIMED(tm, K_UPDATE, s, (k_floor<R><<<gu, kThreads, 0, s>>>(a.patches, a.tasksu, sc, a.d_floors)));
   return cudaGetLastError();
@@ -1110,12 +1195,9 @@ cudaError_t launch_advance(const AdvanceArgs& a, R* scr, R* K, const SolverConst
     if (e != cudaSuccess) return e;
     MHD_TIMED(tm, K_PRED, s, (k_pred<R><<<g1f, bf, kPredSmem<R> * bf, s>>>(d_patches, d_tasks1, scr, sc, K)));
   }
-  constexpr bool inl = kInlineEdges<R>;
-  if (!inl) MHD_TIMED(tm, K_EDGE, s, (k_edge<R><<<g1, kThreads, 0, s>>>(d_patches, d_tasks, scr)));
+  if (!kInlineEdges<R>) MHD_TIMED(tm, K_EDGE, s, (k_edge<R><<<g1, kThreads, 0, s>>>(d_patches, d_tasks, scr)));
   MHD_TIMED(tm, K_FLUX, s, (k_flux<R><<<g1f, bf, 0, s>>>(d_patches, d_tasks1, scr, sc, K)));
-  if (!inl) MHD_TIMED(tm, K_EMF, s, (k_emf<R><<<gu, kThreads, 0, s>>>(d_patches, d_tasksu, scr, sc)));
-  MHD_TIMED(tm, K_UPDATE, s,
-            (k_update<R, inl><<<gu, kThreads, 0, s>>>(d_patches, d_tasksu, scr, sc, K, commit ? 1 : 0)));
+  launch_update<R>(a, scr, K, sc, s);
   if (commit && (a.p_floor > 0.0 || a.rho_floor > 0.0))
     MHD_TIMED(tm, K_UPDATE, s, (k_floor<R><<<gu, kThreads, 0, s>>>(d_patches, d_tasksu, sc, a.d_floors)));
   return cudaGetLastError();

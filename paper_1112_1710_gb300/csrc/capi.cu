@@ -4,6 +4,7 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <cmath>
 #include <array>
 #include <cstdarg>
 #include <cstdio>
@@ -89,7 +90,8 @@ struct mhd_ctx {
   int64_t launches = 0;
   // advance path per element type (index MHD_F64 / MHD_F32) as picked by the
   // autotuner: staged or fused, the fused variant and its z-chunk length (0:
-  // chosen per call); staged until the autotuner measured otherwise
+  // chosen per call); until it measured, pf_by_size decides
+  bool tuned[2] = {false, false};
   bool use_fused[2] = {false, false};
   bool pred_tiled[2] = {false, false};  // staged path: the shared-memory-tiled predictor
   bool use_pf[2] = {false, false};      // the fused primitive / predictor / Riemann pass
@@ -459,6 +461,7 @@ mhd_status mhd_ctx_clone(const mhd_ctx* src, mhd_ctx** out) {
   mhd_status r = mhd_ctx_create(&src->prm, src->device, &c);
   if (r) return r;
   for (int i = 0; i < 2; ++i) {
+    c->tuned[i] = src->tuned[i];
     c->use_fused[i] = src->use_fused[i];
     c->pred_tiled[i] = src->pred_tiled[i];
     c->use_pf[i] = src->use_pf[i];
@@ -617,15 +620,77 @@ void fused_items(const std::vector<DPatch>& dp, int bx, int by, int cz, std::vec
   tasks_for(ccnt, ctasks);
 }
 
+// Extents of the UB+1 region along axis d, and its tiles of at most `cap` cells.
+int pf_extent(const PatchSize& q, int d) { return q.n[d] + 2 * q.k + 2; }
+int64_t pf_tiles(const PatchSize& q, int tx, int ty) {
+  return (int64_t)((pf_extent(q, 0) + tx - 1) / tx) * ((pf_extent(q, 1) + ty - 1) / ty);
+}
+
+// Is an advance that nobody tuned or forced run by the fused pass?  FP64 is
+// bound by its own pipe either way and stays staged.  FP32, staged against fused pass:
+// - Patches advanced with a given dt (serving batches) always take it: a patch gives
+//   the same bits alone and in any batch, so the choice must not depend on the
+//   call's size.  Batches of 65 k cells 91 / 88 us, 512 k 159 / 137, 4 M 898 /
+//   693; a lone 32^3 patch loses 3 us.
+// - Single-level steps that reduce their own CFL dt (which the staged
+//   primitive pass gives for nothing, and the fused pass needs a launch for)
+//   take it from 2,400 cells of UB+1 per SM on, in columns of eight planes or
+//   more: 64^3, 1,890 cells per SM, 72 / 76 us, 72^3, 2,670, 96 / 90, 96^3
+//   184 / 169, 128^3 363 / 318; flat 256^2 x 1 59 / 67.
+// - Calls of a hierarchy (flux-register captures, grown update boxes) stay
+//   staged: the fused pass would bring a coarse step of 64^3 + 3
+//   levels from 80 to 65 ms, but its rounding moves the hierarchy's FP64 dt by 1e-6 over a step.
+//   Tuning such a hierarchy opts in.
+bool pf_by_size(const std::vector<PatchSize>& ps, int dtype, int nsm, int32_t ncap, bool cfl_dt) {
+  if (dtype != MHD_F32 || ncap > 0) return false;
+  int64_t cells = 0;
+  for (const PatchSize& q : ps) {
+    if (q.k > 0) return false;
+    if (pf_extent(q, 2) >= 8) cells += (int64_t)pf_extent(q, 0) * pf_extent(q, 1) * pf_extent(q, 2);
+  }
+  return !cfl_dt || cells >= 2400 * (int64_t)nsm;
+}
+
+// Planes per work item of the fused pass.  The blocks of a call run in rounds
+// of `slots`; a round costs an item's planes and kPfStart planes for its start.
+// The length with the shortest rounds, taking a last round that is part full at
+// half way between its share and a whole one (it runs with less company on its
+// SMs).  128^3 in FP32 (81 tiles of 130 planes, 304 slots): 4 planes 377 us a step,
+// 8 362, 12 348, 16 388, 24 383, 33 451; the rule takes 12.  Hundreds of small
+// patches fill many rounds, and whole columns win.
+int pf_chunk(const std::vector<PatchSize>& ps, int tx, int ty, int slots) {
+  constexpr double kPfStart = 1.6;
+  int zmax = 1;
+  for (const PatchSize& q : ps) zmax = std::max(zmax, pf_extent(q, 2));
+  int best = 0;
+  double best_t = 1e300;
+  for (int cz : {2, 3, 4, 5, 6, 8, 10, 12, 14, 16, 20, 24, 28, 33, 40, 48, 66, 88, 130}) {
+    const int big = std::min(cz, zmax);
+    double planes = 0.0;
+    for (const PatchSize& q : ps)
+      planes += (double)pf_tiles(q, tx, ty) * (pf_extent(q, 2) + kPfStart * ((pf_extent(q, 2) + cz - 1) / cz));
+    const double rounds = planes / ((big + kPfStart) * slots);
+    const double t = (big + kPfStart) * 0.5 * (rounds + std::ceil(rounds));
+    if (t < best_t) {
+      best_t = t;
+      best = cz;
+    }
+    if (cz >= zmax) break;
+  }
+  return best;
+}
+
 // Work items of the fused primitive / predictor / Riemann pass: x-y tiles of
 // at most tx x ty cells over each patch's UB+1 region, the extents along each
-// axis as equal as the cell count allows, and chunks of cz of its planes.
-void pf_items(const std::vector<DPatch>& dp, int tx, int ty, int cz, std::vector<FusedItem>& items) {
+// axis as equal as the cell count allows, and chunks of cz of its planes (0:
+// pf_chunk's).
+void pf_items(const std::vector<PatchSize>& ps, int tx, int ty, int cz, int slots, std::vector<FusedItem>& items) {
   items.clear();
-  for (size_t p = 0; p < dp.size(); ++p) {
-    const DPatch& q = dp[p];
+  if (cz <= 0) cz = pf_chunk(ps, tx, ty, slots);
+  for (size_t p = 0; p < ps.size(); ++p) {
+    const PatchSize& q = ps[p];
     const int lo = q.g - q.k - 1;
-    const int ex = q.n[0] + 2 * q.k + 2, ey = q.n[1] + 2 * q.k + 2, ez = q.n[2] + 2 * q.k + 2;
+    const int ex = pf_extent(q, 0), ey = pf_extent(q, 1), ez = pf_extent(q, 2);
     const int nx = (ex + tx - 1) / tx, ny = (ey + ty - 1) / ty;
     for (int z0 = 0; z0 < ez; z0 += cz)
       for (int j = 0, y0 = 0; j < ny; ++j) {
@@ -668,12 +733,12 @@ std::vector<int32_t> sized_key(const std::vector<PatchSize>& ps, std::initialize
   return key;
 }
 
-mhd_status pf_table(mhd_ctx* c, const std::vector<DPatch>& dp, const std::vector<PatchSize>& ps, const PfVariant& v,
-                    int cz, AdvanceArgs& a) {
-  const std::vector<int32_t> key = sized_key(ps, {v.tx, v.ty, cz});
+mhd_status pf_table(mhd_ctx* c, const std::vector<PatchSize>& ps, const PfVariant& v, int cz, AdvanceArgs& a) {
+  const int slots = v.minb * c->nsm;
+  const std::vector<int32_t> key = sized_key(ps, {v.tx, v.ty, cz, slots});
   return keyed_table<FusedItem>(
       c, TK_PF_ITEMS, key.data(), key.size() * sizeof(int32_t),
-      [&](std::vector<FusedItem>& items) { pf_items(dp, v.tx, v.ty, cz, items); }, &a.pf_items, &a.npf);
+      [&](std::vector<FusedItem>& items) { pf_items(ps, v.tx, v.ty, cz, slots, items); }, &a.pf_items, &a.npf);
 }
 
 mhd_status fused_tables(mhd_ctx* c, const std::vector<DPatch>& dp, const std::vector<PatchSize>& ps,
@@ -780,7 +845,8 @@ static mhd_status scan_captures(mhd_ctx* c, std::vector<DPatch>& dp, const mhd_c
 
 // The advance of mhd_patch_advance; with cfl_dt set (single-level steps, no
 // captures), the step first computes its own CFL dt into *d_dt: inside k_prim
-// for the staged kernels, by the separate reduction before the fused one.
+// for the staged kernels, by k_cfl_step before the fused pass, by the separate
+// reduction before the fused kernel.
 static mhd_status advance_impl(mhd_ctx* c, const mhd_patch_desc* patches, int32_t n, const int32_t* grow,
                         const double* d_dt, const double* dt_scale, const mhd_capture* caps, int32_t ncap,
                         void* stream, bool cfl_dt) {
@@ -793,13 +859,16 @@ static mhd_status advance_impl(mhd_ctx* c, const mhd_patch_desc* patches, int32_
   std::vector<DPatch> dp;
   const int dtype = patches[0].dtype;
   if ((r = advance_patches(c, patches, n, grow, dt_scale, dp))) return r;
+  const std::vector<PatchSize> ps = sizes_of(dp);
   // which advance: the context's (autotuned) choice, or forced staged / fused
   bool fused = c->prm.advance_kernel == 2 || (c->prm.advance_kernel == 0 && c->use_fused[dtype == MHD_F32 ? 1 : 0]);
+  const int di = dtype == MHD_F32 ? 1 : 0;
   const bool pf = !fused && (c->prm.advance_kernel == 4 ||
-                             (c->prm.advance_kernel == 0 && c->use_pf[dtype == MHD_F32 ? 1 : 0]));
-  if (cfl_dt && (fused || pf)) {
-    // neither the fused kernel nor the fused pass has a primitive pass of its
-    // own: the CFL reduction runs first
+                             (c->prm.advance_kernel == 0 &&
+                              (c->tuned[di] ? c->use_pf[di] : pf_by_size(ps, dtype, c->nsm, ncap, cfl_dt))));
+  if (cfl_dt && fused) {
+    // the fused kernel has no primitive pass of its own: the CFL reduction
+    // runs first
     if ((r = mhd_cfl_dt(c, patches, n, nullptr, const_cast<double*>(d_dt), stream))) return r;
     cfl_dt = false;
   }
@@ -822,17 +891,15 @@ static mhd_status advance_impl(mhd_ctx* c, const mhd_patch_desc* patches, int32_
   const size_t es = elem_size(dtype);
   const size_t counter_byte = ((size_t)off * es + 15) / 16 * 16;
   if ((r = ensure_scratch(c, counter_byte + 16))) return r;
-  const int di = dtype == MHD_F32 ? 1 : 0;
   const int shape = c->prm.kernel_shape > 0 ? c->prm.kernel_shape - 1 : pf ? c->pf_variant[di] : c->fused_variant[di];
   if (shape >= (pf ? (di ? kNumPf32 : kNumPf64) : (di ? kNumFused32 : kNumFused64)))
     return fail(c, MHD_EINVAL, "kernel_shape %d is not compiled for this element type", c->prm.kernel_shape);
   AdvanceArgs a{};
   a.nsm = c->nsm;
-  const std::vector<PatchSize> ps = sizes_of(dp);
   if (pf) {
-    const int cz = c->prm.fused_chunk > 0 ? c->prm.fused_chunk : c->fused_chunk[di] > 0 ? c->fused_chunk[di] : 16;
+    const int cz = c->prm.fused_chunk > 0 ? c->prm.fused_chunk : c->fused_chunk[di];
     if ((r = staged_tables(c, ps, es, false, a))) return r;
-    if ((r = pf_table(c, dp, ps, di ? kPfVariants32[shape] : kPfVariants64[shape], cz, a))) return r;
+    if ((r = pf_table(c, ps, di ? kPfVariants32[shape] : kPfVariants64[shape], cz, a))) return r;
   } else if (!fused) {
     if ((r = staged_tables(c, ps, es, true, a))) return r;
     if (c->prm.advance_kernel == 3 || c->pred_tiled[di])
@@ -870,7 +937,7 @@ static mhd_status advance_impl(mhd_ctx* c, const mhd_patch_desc* patches, int32_
   cudaError_t e = run_advance_args(c, dtype, a, (cudaStream_t)stream);
   if (e != cudaSuccess) return cuda_fail(c, e, "patch advance launch");
   // fused: step constants, k_fused, k_commit; staged with the CFL dt: + reset
-  c->launches += (fused ? 3 : pf ? (elem_size(dtype) == 8 ? 4 : 3) : staged_launches(elem_size(dtype)) + (cfl_dt ? 1 : 0)) +
+  c->launches += (fused ? 3 : advance_launches(es, pf, a.emf, a.nblocksu, a.nsm) + (cfl_dt ? (pf ? 2 : 1) : 0)) +
                  (c->prm.p_floor > 0.0 || c->prm.rho_floor > 0.0 ? 1 : 0);
   if (ncap > 0) {
     PackedTasks pc{};
@@ -968,7 +1035,7 @@ mhd_status mhd_autotune_advance(mhd_ctx* c, const mhd_patch_desc* patches, int32
   std::vector<std::pair<int, int>> cand;
   const int npv = dtype == MHD_F32 ? kNumPf32 : kNumPf64;
   for (int sv = 0; sv < npv; ++sv) {
-    std::vector<int> chunks;
+    std::vector<int> chunks{0};  // 0: pf_chunk's choice
     for (int cz : {6, 8, 12, 16, 24, 33}) {
       cz = cz > zmax + 2 ? zmax + 2 : cz;
       if (std::find(chunks.begin(), chunks.end(), cz) == chunks.end()) chunks.push_back(cz);
@@ -1012,7 +1079,7 @@ mhd_status mhd_autotune_advance(mhd_ctx* c, const mhd_patch_desc* patches, int32
     a.commit = false;  // every candidate leaves the patch state as it is
     a.fused = v >= 0;
     if (v <= -3) {
-      r = pf_table(c, dp, ps, dtype == MHD_F32 ? kPfVariants32[-3 - v] : kPfVariants64[-3 - v], cz, a);
+      r = pf_table(c, ps, dtype == MHD_F32 ? kPfVariants32[-3 - v] : kPfVariants64[-3 - v], cz, a);
       a.pf = true;
       a.variant = -3 - v;
     }
@@ -1044,7 +1111,7 @@ mhd_status mhd_autotune_advance(mhd_ctx* c, const mhd_patch_desc* patches, int32
       cudaEventDestroy(e1);
       return cuda_fail(c, e, "autotune run");
     }
-    c->launches += (a.fused ? 3 : a.pf ? (es == 8 ? 4 : 3) : staged_launches(es)) * (reps + 1);
+    c->launches += (a.fused ? 3 : advance_launches(es, a.pf, a.emf, a.nblocksu, a.nsm)) * (reps + 1);
     ms /= reps;
     if (ms < best) {
       best = ms;
@@ -1056,6 +1123,7 @@ mhd_status mhd_autotune_advance(mhd_ctx* c, const mhd_patch_desc* patches, int32
   cudaEventDestroy(e0);
   cudaEventDestroy(e1);
   if (!any) return fail(c, MHD_ECUDA, "autotune: no advance ran on this device");
+  c->tuned[di] = true;
   c->use_fused[di] = bv >= 0;
   c->use_pf[di] = bv <= -3;
   if (bv == -2 || bv == -1) c->pred_tiled[di] = bv == -1;
@@ -1063,7 +1131,7 @@ mhd_status mhd_autotune_advance(mhd_ctx* c, const mhd_patch_desc* patches, int32
   c->pf_variant[di] = bv <= -3 ? -3 - bv : 0;
   c->fused_chunk[di] = bv >= 0 || bv <= -3 ? bcz : 0;
   if (variant_out) *variant_out = bv;
-  if (chunk_out) *chunk_out = bcz;
+  if (chunk_out) *chunk_out = bv <= -3 && bcz == 0 ? zmax + 2 : bcz;  // pf_chunk's choice at each call
   if (ms_out) *ms_out = best;
   return MHD_OK;
 }

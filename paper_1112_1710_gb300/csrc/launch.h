@@ -56,8 +56,8 @@ struct AdvanceArgs {
 
 // Compiled shapes of the fused primitive / predictor / Riemann pass (k_pf):
 // the largest x-y tile and the blocks per SM its registers and shared memory
-// allow (FP32: 16 x 16 at 2, 92 KB; 16 x 12 and 24 x 8 at 3, 71-72 KB;
-// 16 x 8 at 4, 50 KB).
+// allow (FP32: 16 x 16 at 2, 67 KB; 16 x 12 and 24 x 8 at 3, 53-54 KB;
+// 16 x 8 at 4, 38 KB).
 struct PfVariant {
   int tx, ty, minb;
 };
@@ -89,10 +89,23 @@ constexpr int region_m1(size_t) { return 1; }
 constexpr int region_mu(size_t) { return 0; }
 constexpr int region_mu_top(size_t) { return 1; }
 
-// Kernel launches of one staged advance: step constants, k_prim, k_pred,
-// k_flux, k_update, and k_edge and k_emf in FP64 (one more, the dt reset,
-// when k_prim computes the CFL dt).
-inline int staged_launches(size_t elem) { return elem == 8 ? 7 : 5; }
+// Does k_update compute the edge EMFs itself, or read k_emf's planes?  The
+// arithmetic mean is inlined in FP32.  The upwinded EMF reads 12 values an edge and
+// an edge is needed by up to three threads, so FP32 calls of a block or more
+// per SM take k_emf, which computes each edge once from vector loads (149 x 101
+// x 83 cells: k_update 86 -> k_emf + k_update 69 us; 96^3 a step 214 -> 200 us);
+// below, the launch costs what it saves (21 x 18 x 25: 43 against 45 us).
+inline bool update_emf_inline(size_t elem, int emf, int nblocksu, int nsm) {
+  return elem == 4 && (emf == 1 || nblocksu < nsm);
+}
+
+// Kernel launches of one advance (one more, the dt reset, when k_prim computes
+// the CFL dt): staged the step constants, k_prim, k_pred, k_flux, k_update,
+// and k_edge in FP64; the fused pass the step constants, k_pf, k_update; both
+// k_emf where k_update does not compute the edge EMFs.
+inline int advance_launches(size_t elem, bool pf, int emf, int nblocksu, int nsm) {
+  return (pf ? 3 : elem == 8 ? 6 : 5) + (update_emf_inline(elem, emf, nblocksu, nsm) ? 0 : 1);
+}
 
 cudaError_t advance_f64(const AdvanceArgs& a, cudaStream_t s);
 cudaError_t advance_f64c(const AdvanceArgs& a, cudaStream_t s);

@@ -6,134 +6,170 @@
 //
 // A work item is an x-y tile of tx x ty cells (at most TX x TY, the host
 // splits each patch's UB+1 region into tiles of near-equal extents) and a
-// chunk [z0, z1) of its planes.  A block has one thread per tile cell and one
+// chunk [z0, z1) of its planes.  A block has one thread per tile cell, one
 // per cell of the tile's lower x column and lower y row (the left neighbours
-// whose upper face states the tile's lowest faces need); the shared-memory
-// arrays are laid out for the largest tile.  Marching along z,
-// for each plane zc:
-//   1. the primitives W and cell EMFs E^n of plane zc + 1 over the tile grown
-//      by two cells below and one above (the stencil of the predictor and of
-//      the edge averages) go into rings of three planes in shared memory;
-//   2. every thread runs the predictor of its cell on plane zc (limited
-//      slopes, Hancock increment, six predicted face states) and leaves the
-//      states the tile's faces read in shared memory: the lower x, y and z
-//      states of tile cells, the upper x states of the tile and the left
-//      column and the upper y states of the tile and the lower row; the
-//      tile's upper z states stay in registers until the plane's faces are
-//      done and then replace the previous plane's in shared memory;
-//   3. the block's threads take the tile's lower x, y and z faces of plane zc
-//      (the faces of one axis in runs of whole warps): the CT half-step
-//      normal field from edge averages of E^n, the HLLD flux, stored in the
-//      staged layout (vector groups) for k_update and the captures.
-// The predictor and the Riemann solver thus never hold registers at the same
-// time, which keeps the kernel at two to four blocks per SM in FP32 (by tile
-// shape).  Each element is
-// computed with the staged kernels' expressions in the same order (the FP64
-// parity build of this kernel gives the staged, and so the oracle's, bits).
-// Tiles overlap only in the predictor of their lower column and row.
+// whose upper face states the tile's lowest faces need) and up to a warp or
+// two more; the shared-memory arrays are laid out for the largest tile.
+// Marching along z, for each plane zc:
+//   1. every thread runs the predictor of its cell on plane zc (limited
+//      slopes, Hancock increment, six predicted face states) from the rings of
+//      primitives W.  A tile cell keeps its own lower states and its upper z state
+//      in registers; the upper x and y states, which neighbours read, go to
+//      shared memory;
+//   2. the block loads plane zc + 2 into the rings (primitives and cell EMFs E^n
+//      over the tile grown by two cells below and one above), a cell to each
+//      tile thread and the rest to the other threads, and each tile thread takes
+//      its cell's three lower faces: the CT half-step normal field from E^n, the
+//      HLLD flux, stored in the staged layout (vector groups) for k_update and
+//      the captures.
+// A barrier after each.  W has three planes (plane zc - 1 is done with once the
+// predictor has run), E^n four (the faces read zc - 1 to zc + 1).
+//
+// Bound by instruction issue: 244 MB per 128^3 launch, 4% of the DRAM rate.
+// Against a form with one face per thread and turn, every state in shared
+// memory, three barriers a plane, both sides of the fan solved and each face's
+// conserved state computed twice, at 128^3 in FP32: 3,010 -> 2,480 warp
+// instructions per 32 cells, 318 -> 207 us.  Tried and slower: 256 threads with tiles of 15 x 15
+// (the loads lack threads: 368 against 345 us a step), the next plane's reads held
+// in registers across the x face (398 us), one item chain per resident block
+// with equal shares (359 us; neighbouring tiles then run at different planes).
+// Tiles overlap only in the predictor of their lower column and row.  The
+// FP64 parity build keeps the staged expressions and order (the staged, and so
+// the oracle's, bits).
 #pragma once
 
 template <int TX, int TY> struct PfLayout {
   static constexpr int NC = TX * TY;             // tile cells
-  static constexpr int NT = NC + TX + TY;        // threads
+  // threads: the tile's, its lower row's and left column's, in whole warps, and
+  // for the largest tile a warp that only loads
+  static constexpr int NT = (NC + TX + TY + 31) / 32 * 32 + (NC == 256 ? 32 : 0);
   static constexpr int PX = TX + 3, PY = TY + 3; // W / E^n region: x0-2 .. x0+TX
   static constexpr int G = PX * PY;
   static constexpr int NXU = (TX + 1) * TY;      // upper x states: cells x0-1 .. x0+TX-1
   static constexpr int NYU = TX * (TY + 1);      // upper y states: rows y0-1 .. y0+TY-1
   // offsets in elements
   static constexpr int W = 0;                    // [3][8][G]
-  static constexpr int EN = W + 3 * 8 * G;       // [3][3][G]
-  static constexpr int XU = EN + 3 * 3 * G;      // [7][NXU]
+  static constexpr int EN = W + 3 * 8 * G;       // [4][3][G]
+  static constexpr int XU = EN + 4 * 3 * G;      // [7][NXU]
   static constexpr int YU = XU + 7 * NXU;        // [7][NYU]
-  static constexpr int LO = YU + 7 * NYU;        // [3][7][NC] lower x, y, z states (tile cell order)
-  static constexpr int ZU = LO + 3 * 7 * NC;     // [7][NC] upper z states of the previous plane (same)
-  static constexpr int TOTAL = ZU + 7 * NC;
+  static constexpr int TOTAL = YU + 7 * NYU;
 };
 
-// The predictor of one cell from the W ring: the six predicted face states
-// in their faces' rotated frames (7 values each), and the Hancock increment
-// (zero after the second positivity rule's fallback) for the reference EMF.
-template <typename R, int TX, int TY>
+// Limited slope (Half: half of it) of component q along axis d of the cell at
+// ring position s of plane W0 (Wm, Wp: the planes below and above).
+template <typename R, int TX, int TY, bool Half>
+__device__ __forceinline__ R pf_slope(const R* W0, const R* Wm, const R* Wp, int s, int d, int q, R w, int lim) {
+  using L = PfLayout<TX, TY>;
+  const int so = d == 0 ? 1 : L::PX;
+  const R wm = d == 2 ? Wm[q * L::G + s] : W0[q * L::G + s - so];
+  const R wp = d == 2 ? Wp[q * L::G + s] : W0[q * L::G + s + so];
+  return Half ? half_slope(lim, w - wm, wp - w) : limiter(lim, w - wm, wp - w);
+}
+
+// The predictor of one cell from the W ring: put(f, pw) takes the six
+// predicted face states (f = 2 axis + side, primitives in xyz order), again
+// with the cell's own w after the second positivity rule; duk is the Hancock
+// increment (zero after that fallback) for the reference EMF.
+template <typename R, int TX, int TY, typename Put>
 __device__ __forceinline__ void pf_predict(const R* __restrict__ sm, int s, int zc, const SolverConsts<R>& sc,
-                                           const StepDt<R>& st, R (&fs)[6][7], R (&duk)[8], R (&w)[8]) {
+                                           const StepDt<R>& st, R (&duk)[8], R (&w)[8], const Put& put) {
   using L = PfLayout<TX, TY>;
   const R* W0 = sm + L::W + (zc % 3) * 8 * L::G;
   const R* Wm = sm + L::W + ((zc + 2) % 3) * 8 * L::G;
   const R* Wp = sm + L::W + ((zc + 1) % 3) * 8 * L::G;
-  R dw[3][8];
 #pragma unroll
   for (int q = 0; q < 8; ++q) w[q] = W0[q * L::G + s];
-  bool bad = false;
-#pragma unroll
-  for (int d = 0; d < 3; ++d) {
-#pragma unroll
-    for (int q = 0; q < 8; ++q) {
-      R wm, wp;
-      if (d == 0) {
-        wm = W0[q * L::G + s - 1];
-        wp = W0[q * L::G + s + 1];
-      } else if (d == 1) {
-        wm = W0[q * L::G + s - L::PX];
-        wp = W0[q * L::G + s + L::PX];
-      } else {
-        wm = Wm[q * L::G + s];
-        wp = Wp[q * L::G + s];
-      }
-      dw[d][q] = limiter(sc.limiter, w[q] - wm, wp - w[q]);
-    }
-    if (face_rule1(w, dw[d])) bad = true;
-  }
+  bool bad = false, bad2 = false;
   R du[8];
+  if constexpr (sizeof(R) == 4) {
+    // conserved face states computed once, with the flux of their face
+    R u[6][8];
 #pragma unroll
-  for (int q = 0; q < 8; ++q) du[q] = R(0);
+    for (int d = 0; d < 3; ++d) {
+      R h[8], fw[8], fm[8], fp[8];
 #pragma unroll
-  for (int d = 0; d < 3; ++d) {
-    R fwm[8], fwp[8], fm[8], fp[8];
+      for (int q = 0; q < 8; ++q) h[q] = pf_slope<R, TX, TY, true>(W0, Wm, Wp, s, d, q, w[q], sc.limiter);
+      if (face_rule1(w[0], h[0]) || face_rule1(w[4], h[4])) bad = true;
 #pragma unroll
-    for (int q = 0; q < 8; ++q) {
-      fwm[q] = bad ? w[q] : w[q] - R(0.5) * dw[d][q];
-      fwp[q] = bad ? w[q] : w[q] + R(0.5) * dw[d][q];
+      for (int q = 0; q < 8; ++q) fw[q] = w[q] - h[q];
+      cons_flux<true>(d, fw, sc.igm1, u[2 * d], fm);
+#pragma unroll
+      for (int q = 0; q < 8; ++q) fw[q] = w[q] + h[q];
+      cons_flux<true>(d, fw, sc.igm1, u[2 * d + 1], fp);
+#pragma unroll
+      for (int q = 0; q < 8; ++q) {  // the normal-B flux along an axis is zero
+        const R df = q == 5 + d ? R(0) : st.hdtdx[d] * (fp[q] - fm[q]);
+        du[q] = d == 0 ? -df : du[q] - df;
+      }
     }
-    flux_xyz(d, fwp, sc.igm1, fp);
-    flux_xyz(d, fwm, sc.igm1, fm);
+    if (bad) {  // first positivity rule: zero slopes, hence no increment
+      prim2cons(w, sc.igm1, u[0]);
 #pragma unroll
-    for (int q = 0; q < 8; ++q) du[q] = du[q] - st.hdtdx[d] * (fp[q] - fm[q]);
-  }
-  bool bad2 = false;
+      for (int q = 0; q < 8; ++q) {
+        u[1][q] = u[2][q] = u[3][q] = u[4][q] = u[5][q] = u[0][q];
+        du[q] = R(0);
+      }
+    }
 #pragma unroll
-  for (int d = 0; d < 3; ++d) {
-    const int t1 = (d + 1) % 3, t2 = (d + 2) % 3;
+    for (int f = 0; f < 6; ++f) {
+      R pw[8];
 #pragma unroll
-    for (int sd = 0; sd < 2; ++sd) {
+      for (int q = 0; q < 8; ++q) u[f][q] = u[f][q] + du[q];
+      cons2prim(u[f], sc.gm1, pw);
+      if (!(pw[0] > R(0)) || !(pw[4] > R(0))) bad2 = true;
+      put(f, pw);
+    }
+  } else {
+    R dw[3][8];
+#pragma unroll
+    for (int d = 0; d < 3; ++d) {
+#pragma unroll
+      for (int q = 0; q < 8; ++q) dw[d][q] = pf_slope<R, TX, TY, false>(W0, Wm, Wp, s, d, q, w[q], sc.limiter);
+      if (face_rule1(w, dw[d])) bad = true;
+    }
+#pragma unroll
+    for (int q = 0; q < 8; ++q) du[q] = R(0);
+#pragma unroll
+    for (int d = 0; d < 3; ++d) {
+      R fwm[8], fwp[8], fm[8], fp[8];
+#pragma unroll
+      for (int q = 0; q < 8; ++q) {
+        fwm[q] = bad ? w[q] : w[q] - R(0.5) * dw[d][q];
+        fwp[q] = bad ? w[q] : w[q] + R(0.5) * dw[d][q];
+      }
+      flux_xyz(d, fwp, sc.igm1, fp);
+      flux_xyz(d, fwm, sc.igm1, fm);
+#pragma unroll
+      for (int q = 0; q < 8; ++q) du[q] = du[q] - st.hdtdx[d] * (fp[q] - fm[q]);
+    }
+#pragma unroll
+    for (int f = 0; f < 6; ++f) {
+      const int d = f / 2;
       R fw[8], u[8], pw[8];
 #pragma unroll
-      for (int q = 0; q < 8; ++q) fw[q] = bad ? w[q] : (sd ? w[q] + R(0.5) * dw[d][q] : w[q] - R(0.5) * dw[d][q]);
+      for (int q = 0; q < 8; ++q) fw[q] = bad ? w[q] : (f % 2 ? w[q] + R(0.5) * dw[d][q] : w[q] - R(0.5) * dw[d][q]);
       prim2cons(fw, sc.igm1, u);
 #pragma unroll
       for (int q = 0; q < 8; ++q) u[q] = u[q] + du[q];
       cons2prim(u, sc.gm1, pw);
       if (!(pw[0] > R(0)) || !(pw[4] > R(0))) bad2 = true;
-      R* o = fs[2 * d + sd];
-      o[0] = pw[0]; o[1] = pw[1 + d]; o[2] = pw[1 + t1]; o[3] = pw[1 + t2];
-      o[4] = pw[4]; o[5] = pw[5 + t1]; o[6] = pw[5 + t2];
+      put(f, pw);
     }
   }
 #pragma unroll
   for (int q = 0; q < 8; ++q) duk[q] = du[q];
-  if (bad2) {
+  if (bad2) {  // second positivity rule: first order
 #pragma unroll
-    for (int d = 0; d < 3; ++d) {
-      const int t1 = (d + 1) % 3, t2 = (d + 2) % 3;
-#pragma unroll
-      for (int sd = 0; sd < 2; ++sd) {
-        R* o = fs[2 * d + sd];
-        o[0] = w[0]; o[1] = w[1 + d]; o[2] = w[1 + t1]; o[3] = w[1 + t2];
-        o[4] = w[4]; o[5] = w[5 + t1]; o[6] = w[5 + t2];
-      }
-    }
+    for (int f = 0; f < 6; ++f) put(f, w);
 #pragma unroll
     for (int q = 0; q < 8; ++q) duk[q] = R(0);
   }
+}
+
+// The cell EMF E^n_a at ring position s of plane z.
+template <typename R, int TX, int TY> __device__ __forceinline__ R pf_en(const R* __restrict__ sm, int a, int s, int z) {
+  using L = PfLayout<TX, TY>;
+  return sm[L::EN + ((z & 3) * 3 + a) * L::G + s];
 }
 
 // E^n average at the axis-a edge stored at ring position s of plane z (the
@@ -142,77 +178,49 @@ template <typename R, int TX, int TY, int a>
 __device__ __forceinline__ R pf_edge(const R* __restrict__ sm, int s, int z) {
   using L = PfLayout<TX, TY>;
   constexpr int b = (a + 1) % 3, cc = (a + 2) % 3;
-  // ring offsets along x, y (in the plane) and the plane for z
-  const R* E0 = sm + L::EN + (z % 3) * 3 * L::G + a * L::G;
-  const R* Em = sm + L::EN + ((z + 2) % 3) * 3 * L::G + a * L::G;  // plane z - 1
-  const int so[3] = {1, L::PX, 0};
-  // positions of x - sb - sc, x - sc, x - sb, x (the z axis changes plane)
-  R e00, e10, e01, e11;
-  if (b != 2 && cc != 2) {
-    e00 = E0[s - so[b] - so[cc]];
-    e10 = E0[s - so[cc]];
-    e01 = E0[s - so[b]];
-    e11 = E0[s];
-  } else if (b == 2) {  // sb is the z stride
-    e00 = Em[s - so[cc]];
-    e10 = E0[s - so[cc]];
-    e01 = Em[s];
-    e11 = E0[s];
-  } else {  // cc == 2
-    e00 = Em[s - so[b]];
-    e10 = Em[s];
-    e01 = E0[s - so[b]];
-    e11 = E0[s];
-  }
+  constexpr int so[3] = {1, L::PX, 0}, zo[3] = {0, 0, 1};
+  const R e00 = pf_en<R, TX, TY>(sm, a, s - so[b] - so[cc], z - zo[b] - zo[cc]);
+  const R e10 = pf_en<R, TX, TY>(sm, a, s - so[cc], z - zo[cc]);
+  const R e01 = pf_en<R, TX, TY>(sm, a, s - so[b], z - zo[b]);
+  const R e11 = pf_en<R, TX, TY>(sm, a, s, z);
   return Tr<R>::quarter(e00 + e10 + e01 + e11);
 }
 
-// The flux of the axis-d lower face of tile cell c (position fx, fy on plane
-// zc, element x): the CT half-step normal field from edge averages of E^n,
-// the left state from the upper states of the cell below along d and the
-// right state from the cell's own lower state, then HLLD.
+// The difference along axis q of the axis-a edge averages on the two edges of
+// the axis-d lower face of the cell at s (a, d, q distinct).  FP32 takes
+// it from the four cells that do not cancel, half the reads and a rounding
+// less; FP64 from the two averages, as the staged kernels do.
+template <typename R, int TX, int TY, int a, int d, int q>
+__device__ __forceinline__ R pf_edge_diff(const R* __restrict__ sm, int s, int z) {
+  using L = PfLayout<TX, TY>;
+  constexpr int so[3] = {1, L::PX, 0}, zo[3] = {0, 0, 1};
+  if constexpr (sizeof(R) == 4) {
+    const R hi = pf_en<R, TX, TY>(sm, a, s + so[q], z + zo[q]) +
+                 pf_en<R, TX, TY>(sm, a, s + so[q] - so[d], z + zo[q] - zo[d]);
+    const R lo = pf_en<R, TX, TY>(sm, a, s - so[q], z - zo[q]) +
+                 pf_en<R, TX, TY>(sm, a, s - so[q] - so[d], z - zo[q] - zo[d]);
+    return Tr<R>::quarter(hi - lo);
+  } else {
+    return pf_edge<R, TX, TY, a>(sm, s + so[q], z + zo[q]) - pf_edge<R, TX, TY, a>(sm, s, z);
+  }
+}
+
+// The flux of the axis-d lower face of a tile cell (element x, ring position
+// s of plane zc) between the face states lf and rf (7 values in the face's
+// rotated frame): the CT half-step normal field from edge averages of E^n,
+// then HLLD.
 template <typename R, int TX, int TY, int d>
 __device__ __forceinline__ void pf_face(const R* __restrict__ sm, const DPatch& p, const StepDt<R>& st,
-                                        const SolverConsts<R>& sc, R* scr, int64_t x, int fx, int fy, int zc,
-                                        int x0, int y0, int c) {
-  using L = PfLayout<TX, TY>;
+                                        const SolverConsts<R>& sc, R* scr, int64_t x, int s, int zc, const R (&lf)[7],
+                                        const R (&rf)[7]) {
   constexpr int b = (d + 1) % 3, cc = (d + 2) % 3;
-  const int s = (fy - (y0 - 2)) * L::PX + (fx - (x0 - 2));
-  R dEc, dEb;
-  if (d == 0) {
-    dEc = pf_edge<R, TX, TY, 2>(sm, s + L::PX, zc) - pf_edge<R, TX, TY, 2>(sm, s, zc);
-    dEb = pf_edge<R, TX, TY, 1>(sm, s, zc + 1) - pf_edge<R, TX, TY, 1>(sm, s, zc);
-  } else if (d == 1) {
-    dEc = pf_edge<R, TX, TY, 0>(sm, s, zc + 1) - pf_edge<R, TX, TY, 0>(sm, s, zc);
-    dEb = pf_edge<R, TX, TY, 2>(sm, s + 1, zc) - pf_edge<R, TX, TY, 2>(sm, s, zc);
-  } else {
-    dEc = pf_edge<R, TX, TY, 1>(sm, s + 1, zc) - pf_edge<R, TX, TY, 1>(sm, s, zc);
-    dEb = pf_edge<R, TX, TY, 0>(sm, s + L::PX, zc) - pf_edge<R, TX, TY, 0>(sm, s, zc);
-  }
+  const R dEc = pf_edge_diff<R, TX, TY, cc, d, b>(sm, s, zc);
+  const R dEb = pf_edge_diff<R, TX, TY, b, d, cc>(sm, s, zc);
   const R bh = ((const R*)p.B[d])[x] - (st.hdtdx[b] * dEc - st.hdtdx[cc] * dEb);
-  const R* left;
-  int lstride;
-  if (d == 0) {
-    left = sm + L::XU + (fx - x0) + (fy - y0) * (TX + 1);   // cell fx - 1 in XU
-    lstride = L::NXU;
-  } else if (d == 1) {
-    left = sm + L::YU + (fy - y0) * TX + (fx - x0);         // row fy - 1 in YU
-    lstride = L::NYU;
-  } else {
-    left = sm + L::ZU + c;                                  // plane zc - 1
-    lstride = L::NC;
-  }
-  const R* right = sm + L::LO + d * 7 * L::NC + c;
-  R Lf[8], Rf[8];
-#pragma unroll
-  for (int q = 0; q < 7; ++q) {
-    Lf[q < 5 ? q : q + 1] = left[q * lstride];
-    Rf[q < 5 ? q : q + 1] = right[q * L::NC];
-  }
-  Lf[5] = R(0);
-  Rf[5] = R(0);
+  const R Lf[8] = {lf[0], lf[1], lf[2], lf[3], lf[4], R(0), lf[5], lf[6]};
+  const R Rf[8] = {rf[0], rf[1], rf[2], rf[3], rf[4], R(0), rf[5], rf[6]};
   R fr[8], f[8], upw;
-  hlld<R, kFastRecip>(Lf, Rf, bh, sc.gamma, sc.igm1, sc.eps_up, sc.emf != 1, fr, &upw);
+  hlld_side<R, kFastRecip>(Lf, Rf, bh, sc.gamma, sc.igm1, sc.eps_up, sc.emf != 1, fr, &upw);
   rot_out(d, fr, f);
   f[5 + d] = upw;
   VecIO<R>::store8(arr(scr, p, SC_F + d * 8), p.snelem, x, f);
@@ -249,30 +257,25 @@ __global__ void __launch_bounds__(PfLayout<TX, TY>::NT, MINB)
   }
   // inside UB+1: the predictor is defined there
   const bool act = t < nc + tx + ty && cx >= lo - 1 && cx <= hix + 1 && cy >= lo - 1 && cy <= hiy + 1;
+  // this thread's lower faces, on planes where the axis allows
+  const bool facet = tile && cx <= hix + 1 && cy <= hiy + 1;
   const int s = (cy - (y0 - 2)) * L::PX + (cx - (x0 - 2));
   const int zstart = z0 - 1 >= lo - 1 ? z0 - 1 : z0;
   const int64_t s1 = p.s1, s2 = p.s2;
-  // fills the W / E^n ring slot of plane zl over x0-2 .. x0+tx, y0-2 ..
-  // y0+ty, clipped to UB+2
-  auto load_plane = [&](int zl) {
+  const int rx = tx + 3, nr = rx * (ty + 3);
+  // primitives and E^n of the ring cells rr, rr + step, ... of plane zl
+  auto load_cells = [&](int zl, int rr, int step) {
+    if (zl < lo - 2 || zl > hiz + 2) return;
     R* W = sm + L::W + (zl % 3) * 8 * L::G;
-    R* En = sm + L::EN + (zl % 3) * 3 * L::G;
-    bool bad = false;
-    const int rx = tx + 3;
-    for (int rr = t; rr < rx * (ty + 3); rr += L::NT) {
-      const int lx = rr % rx, ly = rr / rx;
+    R* En = sm + L::EN + (zl & 3) * 3 * L::G;
+    for (; rr < nr; rr += step) {
+      int lx;
+      const int ly = divmod24(rr, rx, lx);
       const int r = ly * L::PX + lx;
       const int gx = x0 - 2 + lx, gy = y0 - 2 + ly;
-      if (gx < lo - 2 || gx > hix + 2 || gy < lo - 2 || gy > hiy + 2 || zl < lo - 2 || zl > hiz + 2) continue;
-      const int64_t x = (int64_t)gx + (int64_t)gy * s1 + (int64_t)zl * s2;
-      R u[8];
-#pragma unroll
-      for (int q = 0; q < 5; ++q) u[q] = ((const R*)p.U[q])[x];
-      u[5] = Tr<R>::half(((const R*)p.B[0])[x] + ((const R*)p.B[0])[x + 1]);
-      u[6] = Tr<R>::half(((const R*)p.B[1])[x] + ((const R*)p.B[1])[x + s1]);
-      u[7] = Tr<R>::half(((const R*)p.B[2])[x] + ((const R*)p.B[2])[x + s2]);
+      if (gx < lo - 2 || gx > hix + 2 || gy < lo - 2 || gy > hiy + 2) continue;
       R w[8];
-      cons2prim(u, sc.gm1, w);
+      load_prim(p, (int64_t)gx + (int64_t)gy * s1 + (int64_t)zl * s2, sc, w);
       if (sc.rho_floor > R(0) && !(w[0] >= sc.rho_floor)) w[0] = sc.rho_floor;
       if (sc.p_floor > R(0) && !(w[4] >= sc.p_floor)) w[4] = sc.p_floor;
 #pragma unroll
@@ -282,86 +285,72 @@ __global__ void __launch_bounds__(PfLayout<TX, TY>::NT, MINB)
         const int b = (a + 1) % 3, cc = (a + 2) % 3;
         En[a * L::G + r] = w[1 + cc] * w[5 + b] - w[1 + b] * w[5 + cc];
       }
-      if (!(w[0] > R(0)) || !(w[4] > R(0))) bad = true;
+      if (!(w[0] > R(0)) || !(w[4] > R(0))) raise_status(status, -4);
     }
-    if (bad) raise_status(status, -4);
   };
-  load_plane(zstart - 1);
-  load_plane(zstart);
-  R zup[7];                                  // this tile cell's upper z state on plane zc
+  for (int zl = zstart - 1; zl <= zstart + 1; ++zl) load_cells(zl, t, L::NT);
+  __syncthreads();
+  R zlow[7];  // this tile cell's upper z state on plane zc - 1
 #pragma unroll
-  for (int q = 0; q < 7; ++q) zup[q] = R(0);
+  for (int q = 0; q < 7; ++q) zlow[q] = R(0);
   for (int zc = zstart; zc < z1; ++zc) {
-    load_plane(zc + 1);
-    __syncthreads();
-    // 2. predictor of this thread's cell on plane zc
+    // predictor of this thread's cell on plane zc; a tile cell keeps its
+    // lower states and its upper z state
+    R own[3][7], zup[7];
+#pragma unroll
+    for (int q = 0; q < 7; ++q) zup[q] = own[0][q] = own[1][q] = own[2][q] = R(0);
     if (act) {
-      R fs[6][7], duk[8], w[8];
-      pf_predict<R, TX, TY>(sm, s, zc, sc, st, fs, duk, w);
-      if (tile) {
-        const int c = t;
+      R duk[8], w[8];
+      R* const xu = sm + L::XU + (cy - y0) * (TX + 1) + (cx - (x0 - 1));
+      R* const yu = sm + L::YU + (cy - (y0 - 1)) * TX + (cx - x0);
+      const bool px = cy >= y0, py = cx >= x0;  // not the lower row, not the left column
+      pf_predict<R, TX, TY>(sm, s, zc, sc, st, duk, w, [&](int f, const R (&pw)[8]) {
+        const int d = f >> 1, t1 = (d + 1) % 3, t2 = (d + 2) % 3;
+        const R v[7] = {pw[0], pw[1 + d], pw[1 + t1], pw[1 + t2], pw[4], pw[5 + t1], pw[5 + t2]};
+        if (f == 1) {
+          if (px) {
 #pragma unroll
-        for (int d = 0; d < 3; ++d)
-#pragma unroll
-          for (int q = 0; q < 7; ++q) sm[L::LO + (d * 7 + q) * L::NC + c] = fs[2 * d][q];
-#pragma unroll
-        for (int q = 0; q < 7; ++q) zup[q] = fs[5][q];
-        if (sc.emf != 1 && zc >= z0) {
-          // reference cell EMF from U^{n+1/2}, read by the upwinded EMF average
-          const int64_t x = (int64_t)cx + (int64_t)cy * s1 + (int64_t)zc * s2;
-          R uc[8], uh[8];
-          prim2cons(w, sc.igm1, uc);
-#pragma unroll
-          for (int q = 0; q < 8; ++q) uh[q] = uc[q] + duk[q];
-          R ir = Tr<R>::div(R(1), uh[0]);
-          R v[3] = {uh[1] * ir, uh[2] * ir, uh[3] * ir};
-#pragma unroll
-          for (int a = 0; a < 3; ++a) {
-            const int b = (a + 1) % 3, cc = (a + 2) % 3;
-            arr(scr, p, SC_ER + a)[x] = v[cc] * uh[5 + b] - v[b] * uh[5 + cc];
+            for (int q = 0; q < 7; ++q) xu[q * L::NXU] = v[q];
           }
+        } else if (f == 3) {
+          if (py) {
+#pragma unroll
+            for (int q = 0; q < 7; ++q) yu[q * L::NYU] = v[q];
+          }
+        } else {
+#pragma unroll
+          for (int q = 0; q < 7; ++q) (f == 5 ? zup : own[d])[q] = v[q];
         }
-      }
-      // upper x state: tile cells and the left column; upper y state: tile
-      // cells and the lower row
-      if (cx < x0 + TX && cy >= y0) {
-        const int ix = (cy - y0) * (TX + 1) + (cx - (x0 - 1));
-#pragma unroll
-        for (int q = 0; q < 7; ++q) sm[L::XU + q * L::NXU + ix] = fs[1][q];
-      }
-      if (cy < y0 + TY && cx >= x0) {
-        const int iy = (cy - (y0 - 1)) * TX + (cx - x0);
-#pragma unroll
-        for (int q = 0; q < 7; ++q) sm[L::YU + q * L::NYU + iy] = fs[3][q];
+      });
+      if (tile && sc.emf != 1 && zc >= z0) {
+        // reference cell EMF from U^{n+1/2}, read by the upwinded EMF average
+        const int64_t x = (int64_t)cx + (int64_t)cy * s1 + (int64_t)zc * s2;
+        reference_emf(p, x, scr, sc, w, duk);
       }
     }
     __syncthreads();
-    // 3. the tile's lower faces on plane zc, axis-major, each axis's run
-    // padded to whole warps (warp-uniform axis)
-    if (zc >= z0) {
-      const int ncp = (nc + 31) & ~31;
-      for (int task = t; task < 3 * ncp; task += L::NT) {
-        const int d = task / ncp, c = task - d * ncp;
-        if (c >= nc) continue;
-        const int fx = x0 + c % tx, fy = y0 + c / tx;
-        if (fx > hix + 1 || fy > hiy + 1) continue;
-        if ((d == 0 ? fx : d == 1 ? fy : zc) < lo) continue;
-        if (d == 2 && zc <= zstart) continue;   // no upper z state of plane zc - 1
-        const int64_t x = (int64_t)fx + (int64_t)fy * s1 + (int64_t)zc * s2;
-        if (d == 0)
-          pf_face<R, TX, TY, 0>(sm, p, st, sc, scr, x, fx, fy, zc, x0, y0, c);
-        else if (d == 1)
-          pf_face<R, TX, TY, 1>(sm, p, st, sc, scr, x, fx, fy, zc, x0, y0, c);
-        else
-          pf_face<R, TX, TY, 2>(sm, p, st, sc, scr, x, fx, fy, zc, x0, y0, c);
-      }
-    }
-    // the next plane's load and predictor overwrite the ring slot and the
-    // states this plane's faces read
-    __syncthreads();
-    if (tile) {
+    // the faces of plane zc, and the ring's next plane
+    const bool next = zc + 1 < z1;
+    const bool faces = facet && zc >= z0;
+    const int64_t x = (int64_t)cx + (int64_t)cy * s1 + (int64_t)zc * s2;
+    if (next) load_cells(zc + 2, t, tile ? nr : L::NT - nc);
+    if (faces && zc >= lo && zc > zstart) pf_face<R, TX, TY, 2>(sm, p, st, sc, scr, x, s, zc, zlow, own[2]);
+    R left[7];
+    if (faces && cx >= lo) {
+      const R* xu = sm + L::XU + (cy - y0) * (TX + 1) + (cx - x0);  // cell cx - 1
 #pragma unroll
-      for (int q = 0; q < 7; ++q) sm[L::ZU + q * L::NC + t] = zup[q];
+      for (int q = 0; q < 7; ++q) left[q] = xu[q * L::NXU];
+      pf_face<R, TX, TY, 0>(sm, p, st, sc, scr, x, s, zc, left, own[0]);
     }
+    if (faces && cy >= lo) {
+      const R* yu = sm + L::YU + (cy - y0) * TX + (cx - x0);        // row cy - 1
+#pragma unroll
+      for (int q = 0; q < 7; ++q) left[q] = yu[q * L::NYU];
+      pf_face<R, TX, TY, 1>(sm, p, st, sc, scr, x, s, zc, left, own[1]);
+    }
+#pragma unroll
+    for (int q = 0; q < 7; ++q) zlow[q] = zup[q];
+    // the next plane's predictor reads the ring and replaces the upper states
+    __syncthreads();
   }
 }

@@ -212,8 +212,12 @@ template <bool FR, typename R> __device__ __forceinline__ R recip(R b) {
   else return R(0);
 }
 
-// FP32 HLLD (hlld64's formulas and reciprocal form): both sides of the fan in
-// full, every region's flux from F* = F + S (U* - U).
+// FP32 HLLD of the staged and the fused kernels (hlld_side's formulas and
+// reciprocal form): both sides of the fan in full, every region's flux from
+// F* = F + S (U* - U).  Those kernels move 200 bytes a face and wait for
+// memory either way (k_flux 115 against 109 us at 128^3), and their rounding
+// is kept: a hierarchy's time step amplifies it (pf_by_size).  The fused pass
+// takes hlld_side.
 template <typename R>
 __device__ __forceinline__ void hlld32(const R* L, const R* Rr, R bn, R gamma, R igm1, R eps_up,
                                        R* f, R* upw) {
@@ -361,7 +365,7 @@ __device__ __forceinline__ void hlld32(const R* L, const R* Rr, R bn, R gamma, R
 // S_M = u (a plain reciprocal would turn x/x into x (1/x), off by an ulp,
 // and give a 2D problem a z-field of rounding noise).
 template <typename R, bool FR = false>
-__device__ __forceinline__ void hlld64(const R* L, const R* Rr, R bn, R gamma, R igm1, R eps_up, bool up,
+__device__ __forceinline__ void hlld_side(const R* L, const R* Rr, R bn, R gamma, R igm1, R eps_up, bool up,
                                      R* f, R* upw) {
   using T = Tr<R>;
   R rl = L[0], ul = L[1], vl = L[2], wl_ = L[3], pl = L[4], byl = L[6], bzl = L[7];
@@ -458,9 +462,16 @@ __device__ __forceinline__ void hlld64(const R* L, const R* Rr, R bn, R gamma, R
   const R es = qdiv<FR>(((sd * e - pt * u) + pts * sm) + bn * (vb - vbs), sS, isS);
 
   R sqrl, sqrr, ab;
-  sqrl = T::sqrt_(rls);
-  sqrr = T::sqrt_(rrs);
-  ab = T::div(T::abs(bn), left ? sqrl : sqrr);
+  if constexpr (sizeof(R) == 4) {  // one reciprocal root gives the root and the quotient
+    const R isl = T::rsqrt_(rls), isr = T::rsqrt_(rrs);
+    sqrl = rls * isl;
+    sqrr = rrs * isr;
+    ab = T::abs(bn) * (left ? isl : isr);
+  } else {
+    sqrl = T::sqrt_(rls);
+    sqrr = T::sqrt_(rrs);
+    ab = T::div(T::abs(bn), left ? sqrl : sqrr);
+  }
   const R Ss = left ? sm - ab : sm + ab;
 
   const R mxs = rs * sm;
@@ -535,7 +546,7 @@ template <typename R, bool FR = false>
 __device__ __forceinline__ void hlld(const R* L, const R* Rr, R bn, R gamma, R igm1, R eps_up, bool up, R* f,
                                      R* upw) {
   if constexpr (sizeof(R) == 4) hlld32(L, Rr, bn, gamma, igm1, eps_up, f, upw);
-  else hlld64<R, FR>(L, Rr, bn, gamma, igm1, eps_up, up, f, upw);
+  else hlld_side<R, FR>(L, Rr, bn, gamma, igm1, eps_up, up, f, upw);
 }
 
 }  // namespace mhd
