@@ -97,9 +97,8 @@ typedef struct {
                         fused (about 1.25x faster; differs from 0 by rounding) */
   int32_t advance_kernel; /* 0: the context's choice (what mhd_autotune_advance
                         measured fastest; before that the fused pass for
-                        MHD_F32 calls without captures and grown boxes, in
-                        mhd_patch_step_cfl only if the patches fill the
-                        device, else the staged kernels);
+                        MHD_F32 calls of mhd_patch_advance without captures
+                        and grown boxes, else the staged kernels);
                         1: the staged kernels (one launch per stage,
                         intermediates in the scratch arena; the predictor
                         tiled in shared memory if the autotuner chose it);

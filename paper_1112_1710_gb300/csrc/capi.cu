@@ -90,7 +90,7 @@ struct mhd_ctx {
   int64_t launches = 0;
   // advance path per element type (index MHD_F64 / MHD_F32) as picked by the
   // autotuner: staged or fused, the fused variant and its z-chunk length (0:
-  // chosen per call); until it measured, pf_by_size decides
+  // chosen per call); until it measured, pf_untuned decides
   bool tuned[2] = {false, false};
   bool use_fused[2] = {false, false};
   bool pred_tiled[2] = {false, false};  // staged path: the shared-memory-tiled predictor
@@ -632,23 +632,16 @@ int64_t pf_tiles(const PatchSize& q, int tx, int ty) {
 //   the same bits alone and in any batch, so the choice must not depend on the
 //   call's size.  Batches of 65 k cells 91 / 88 us, 512 k 159 / 137, 4 M 898 /
 //   693; a lone 32^3 patch loses 3 us.
-// - Single-level steps that reduce their own CFL dt (which the staged
-//   primitive pass gives for nothing, and the fused pass needs a launch for)
-//   take it from 2,400 cells of UB+1 per SM on, in columns of eight planes or
-//   more: 64^3, 1,890 cells per SM, 72 / 76 us, 72^3, 2,670, 96 / 90, 96^3
-//   184 / 169, 128^3 363 / 318; flat 256^2 x 1 59 / 67.
-// - Calls of a hierarchy (flux-register captures, grown update boxes) stay
-//   staged: the fused pass would bring a coarse step of 64^3 + 3
-//   levels from 80 to 65 ms, but its rounding moves the hierarchy's FP64 dt by 1e-6 over a step.
-//   Tuning such a hierarchy opts in.
-bool pf_by_size(const std::vector<PatchSize>& ps, int dtype, int nsm, int32_t ncap, bool cfl_dt) {
-  if (dtype != MHD_F32 || ncap > 0) return false;
-  int64_t cells = 0;
-  for (const PatchSize& q : ps) {
+// - Steps that reduce their own CFL dt and calls of a hierarchy (flux-register
+//   captures, grown update boxes) stay staged: the fused pass would bring a
+//   128^3 step from 363 to 318 us and a coarse step of 64^3 + 3 levels from 80
+//   to 65 ms, but its FP32 rounding moves the FP64 dt that follows from the state
+//   by up to 1e-5.  Tuning a context opts in.
+bool pf_untuned(const std::vector<PatchSize>& ps, int dtype, int32_t ncap, bool cfl_dt) {
+  if (dtype != MHD_F32 || ncap > 0 || cfl_dt) return false;
+  for (const PatchSize& q : ps)
     if (q.k > 0) return false;
-    if (pf_extent(q, 2) >= 8) cells += (int64_t)pf_extent(q, 0) * pf_extent(q, 1) * pf_extent(q, 2);
-  }
-  return !cfl_dt || cells >= 2400 * (int64_t)nsm;
+  return true;
 }
 
 // Planes per work item of the fused pass.  The blocks of a call run in rounds
@@ -865,7 +858,7 @@ static mhd_status advance_impl(mhd_ctx* c, const mhd_patch_desc* patches, int32_
   const int di = dtype == MHD_F32 ? 1 : 0;
   const bool pf = !fused && (c->prm.advance_kernel == 4 ||
                              (c->prm.advance_kernel == 0 &&
-                              (c->tuned[di] ? c->use_pf[di] : pf_by_size(ps, dtype, c->nsm, ncap, cfl_dt))));
+                              (c->tuned[di] ? c->use_pf[di] : pf_untuned(ps, dtype, ncap, cfl_dt))));
   if (cfl_dt && fused) {
     // the fused kernel has no primitive pass of its own: the CFL reduction
     // runs first

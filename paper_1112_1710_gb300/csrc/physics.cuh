@@ -216,7 +216,7 @@ template <bool FR, typename R> __device__ __forceinline__ R recip(R b) {
 // reciprocal form): both sides of the fan in full, every region's flux from
 // F* = F + S (U* - U).  Those kernels move 200 bytes a face and wait for
 // memory either way (k_flux 115 against 109 us at 128^3), and their rounding
-// is kept: a hierarchy's time step amplifies it (pf_by_size).  The fused pass
+// is kept: a hierarchy's time step amplifies it (pf_untuned).  The fused pass
 // takes hlld_side.
 template <typename R>
 __device__ __forceinline__ void hlld32(const R* L, const R* Rr, R bn, R gamma, R igm1, R eps_up,
