@@ -67,7 +67,11 @@ __device__ __forceinline__ int flag_exact(const DPatch& p, int64_t x, double gm1
 // within 9 eps, me within 8 eps mb where mb = (sum of the squared means of
 // |B| of the two faces) / 2 >= me, and E, two subtractions, gamma - 1 and
 // their product add 7 eps of |E| + ke + mb at most: 16 eps gm1 (|E| + ke + mb),
-// taken as 24.  Outside [1e-30, 1e30] the bound is infinite.
+// taken as 24.  Outside [1e-30, 1e30] the bound is infinite.  A result below
+// 2^-126 is within 2^-150 instead, so ke is the sum of m (m / rho), whose
+// underflow stays an absolute error of a few 2^-150 (flag_side's 1e-37 covers
+// it); squares of momenta below 1e-19 would lose digits that 1 / rho then
+// multiplies by up to 1e30.
 struct FlagCell {
   float r, p, d;
 };
@@ -79,7 +83,8 @@ template <typename R> __device__ __forceinline__ FlagCell flag_cell(const DPatch
   const float z0 = (float)((const R*)p.B[2])[x], z1 = (float)((const R*)p.B[2])[x + p.s2];
   const float bx = 0.5f * (x0 + x1), by = 0.5f * (y0 + y1), bz = 0.5f * (z0 + z1);
   const float ax = 0.5f * (fabsf(x0) + fabsf(x1)), ay = 0.5f * (fabsf(y0) + fabsf(y1)), az = 0.5f * (fabsf(z0) + fabsf(z1));
-  const float ke = 0.5f * (mx * mx + my * my + mz * mz) * (1.0f / rho);
+  const float ir = 1.0f / rho;
+  const float ke = 0.5f * (mx * (mx * ir) + my * (my * ir) + mz * (mz * ir));
   const float me = 0.5f * (bx * bx + by * by + bz * bz), mb = 0.5f * (ax * ax + ay * ay + az * az);
   const float S = fabsf(E) + fabsf(ke) + mb;
   FlagCell c;
