@@ -110,8 +110,10 @@ typedef struct {
                         Riemann fluxes over x-y tiles marching along z, the
                         predicted face states kept on chip), then the staged
                         EMF and update kernels.  All compute every element
-                        with the same expressions (in MHD_F32 the fused pass
-                        to rounding); a call whose captures need
+                        with the same expressions: the same bits from all of
+                        them in the MHD_F64 parity build and from 1 and 4 in
+                        MHD_F32; elsewhere they differ by rounding;
+                        a call whose captures need
                         face fluxes outside the update box runs staged (2) or
                         takes them from the fused pass's flux planes (4).   */
   int32_t fused_chunk; /* z-planes per work item of the fused kernel (2) or

@@ -763,7 +763,7 @@ __device__ __forceinline__ void flux_face(const DPatch& p, int patch, const Cell
   VecIO<R>::load7(arr(scr, p, SC_WF + (d * 2 + 0) * 8), p.snelem, x, vr);
   const R L[8] = {vl[0], vl[1], vl[2], vl[3], vl[4], R(0), vl[5], vl[6]};
   const R Rr[8] = {vr[0], vr[1], vr[2], vr[3], vr[4], R(0), vr[5], vr[6]};
-  hlld<R, kFastRecip>(L, Rr, bh, sc.gamma, sc.igm1, sc.eps_up, sc.emf != 1, fr, &upw);
+  hlld<R, kFastRecip>(d, L, Rr, bh, sc.gamma, sc.igm1, sc.eps_up, sc.emf != 1, fr, &upw);
   rot_out(d, fr, f);
   f[5 + d] = upw;
   VecIO<R>::store8(arr(scr, p, SC_F + d * 8), p.snelem, x, f);

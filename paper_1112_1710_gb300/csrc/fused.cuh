@@ -239,7 +239,7 @@ __device__ __forceinline__ void face_flux(const R* wl, const R* wr, R bh, const 
   R L[8], Rr[8], fr[8], upw;
   rot_in(d, wl, L);
   rot_in(d, wr, Rr);
-  hlld<R, kFastRecip>(L, Rr, bh, sc.gamma, sc.igm1, sc.eps_up, sc.emf != 1, fr, &upw);
+  hlld<R, kFastRecip>(d, L, Rr, bh, sc.gamma, sc.igm1, sc.eps_up, sc.emf != 1, fr, &upw);
   rot_out(d, fr, f);
   f[5 + d] = upw;
 }

@@ -25,17 +25,20 @@
 // A barrier after each.  W has three planes (plane zc - 1 is done with once the
 // predictor has run), E^n four (the faces read zc - 1 to zc + 1).
 //
-// Bound by instruction issue: 244 MB per 128^3 launch, 4% of the DRAM rate.
-// Against a form with one face per thread and turn, every state in shared
-// memory, three barriers a plane, both sides of the fan solved and each face's
-// conserved state computed twice, at 128^3 in FP32: 3,010 -> 2,480 warp
-// instructions per 32 cells, 318 -> 207 us.  Tried and slower: 256 threads with tiles of 15 x 15
+// Bound by instruction issue (59% of the slots at 17 warps per SM): 240 MB per
+// 128^3 launch in FP32, 13% of the copy rate.  Both types keep the staged
+// kernels' expressions, order and bits: which kernels advance a call depends on its
+// captures, update boxes and size, and neighbouring patches in different
+// calls have to agree on their shared faces.  2,627 warp instructions per 32
+// cells and 266 us at 128^3 in FP32, where k_prim, k_pred and k_flux take 276
+// us and move 1.28 GB.  FP32 expressions of its own (conserved face states
+// shared between a face's flux and its predicted state, the star state's physical flux,
+// four of E^n a face) took 2,480 and 207 us, but a state that differs by rounding.
+// Tried and slower, in that form: 256 threads with tiles of 15 x 15
 // (the loads lack threads: 368 against 345 us a step), the next plane's reads held
 // in registers across the x face (398 us), one item chain per resident block
 // with equal shares (359 us; neighbouring tiles then run at different planes).
-// Tiles overlap only in the predictor of their lower column and row.  The
-// FP64 parity build keeps the staged expressions and order (the staged, and so
-// the oracle's, bits).
+// Tiles overlap only in the predictor of their lower column and row.
 #pragma once
 
 template <int TX, int TY> struct PfLayout {
@@ -55,15 +58,24 @@ template <int TX, int TY> struct PfLayout {
   static constexpr int TOTAL = YU + 7 * NYU;
 };
 
-// Limited slope (Half: half of it) of component q along axis d of the cell at
-// ring position s of plane W0 (Wm, Wp: the planes below and above).
-template <typename R, int TX, int TY, bool Half>
+// The value of x, which the compiler does not see through.  The staged kernels
+// pass slopes and face states through memory; here they stay in registers, where
+// FP32 multiply-adds would be contracted across them and the bits would differ.
+__device__ __forceinline__ float opaque(float x) {
+  asm("" : "+f"(x));
+  return x;
+}
+__device__ __forceinline__ double opaque(double x) { return x; }  // (the contracted FP64 build may)
+
+// Limited slope of component q along axis d of the cell at ring position s of
+// plane W0 (Wm, Wp: the planes below and above).
+template <typename R, int TX, int TY>
 __device__ __forceinline__ R pf_slope(const R* W0, const R* Wm, const R* Wp, int s, int d, int q, R w, int lim) {
   using L = PfLayout<TX, TY>;
   const int so = d == 0 ? 1 : L::PX;
   const R wm = d == 2 ? Wm[q * L::G + s] : W0[q * L::G + s - so];
   const R wp = d == 2 ? Wp[q * L::G + s] : W0[q * L::G + s + so];
-  return Half ? half_slope(lim, w - wm, wp - w) : limiter(lim, w - wm, wp - w);
+  return limiter(lim, w - wm, wp - w);
 }
 
 // The predictor of one cell from the W ring: put(f, pw) takes the six
@@ -80,81 +92,54 @@ __device__ __forceinline__ void pf_predict(const R* __restrict__ sm, int s, int 
 #pragma unroll
   for (int q = 0; q < 8; ++q) w[q] = W0[q * L::G + s];
   bool bad = false, bad2 = false;
-  R du[8];
-  if constexpr (sizeof(R) == 4) {
-    // conserved face states computed once, with the flux of their face
-    R u[6][8];
+  R du[8], dw[3][8];
 #pragma unroll
-    for (int d = 0; d < 3; ++d) {
-      R h[8], fw[8], fm[8], fp[8];
+  for (int d = 0; d < 3; ++d) {
 #pragma unroll
-      for (int q = 0; q < 8; ++q) h[q] = pf_slope<R, TX, TY, true>(W0, Wm, Wp, s, d, q, w[q], sc.limiter);
-      if (face_rule1(w[0], h[0]) || face_rule1(w[4], h[4])) bad = true;
+    for (int q = 0; q < 8; ++q) dw[d][q] = opaque(pf_slope<R, TX, TY>(W0, Wm, Wp, s, d, q, w[q], sc.limiter));
+    if (face_rule1(w, dw[d])) bad = true;
+  }
 #pragma unroll
-      for (int q = 0; q < 8; ++q) fw[q] = w[q] - h[q];
-      cons_flux<true>(d, fw, sc.igm1, u[2 * d], fm);
+  for (int q = 0; q < 8; ++q) du[q] = R(0);
+  if (bad) {
+    // first positivity rule: zero slopes (24 selects, where selecting w for each
+    // face state takes 96; the increment is then +0 and the states are U(w))
 #pragma unroll
-      for (int q = 0; q < 8; ++q) fw[q] = w[q] + h[q];
-      cons_flux<true>(d, fw, sc.igm1, u[2 * d + 1], fp);
+    for (int d = 0; d < 3; ++d)
 #pragma unroll
-      for (int q = 0; q < 8; ++q) {  // the normal-B flux along an axis is zero
-        const R df = q == 5 + d ? R(0) : st.hdtdx[d] * (fp[q] - fm[q]);
-        du[q] = d == 0 ? -df : du[q] - df;
-      }
+      for (int q = 0; q < 8; ++q) dw[d][q] = R(0);
+  }
+#pragma unroll
+  for (int d = 0; d < 3; ++d) {
+    R fwm[8], fwp[8], fm[8], fp[8];
+#pragma unroll
+    for (int q = 0; q < 8; ++q) {
+      fwm[q] = w[q] - R(0.5) * dw[d][q];
+      fwp[q] = w[q] + R(0.5) * dw[d][q];
     }
-    if (bad) {  // first positivity rule: zero slopes, hence no increment
-      prim2cons(w, sc.igm1, u[0]);
+    flux_xyz(d, fwp, sc.igm1, fp);
+    flux_xyz(d, fwm, sc.igm1, fm);
 #pragma unroll
-      for (int q = 0; q < 8; ++q) {
-        u[1][q] = u[2][q] = u[3][q] = u[4][q] = u[5][q] = u[0][q];
-        du[q] = R(0);
-      }
-    }
+    for (int q = 0; q < 8; ++q) du[q] = du[q] - st.hdtdx[d] * (fp[q] - fm[q]);
+  }
+  // the face states anew, as the staged predictor takes them (not merged with
+  // the flux's, which would change what is contracted)
 #pragma unroll
-    for (int f = 0; f < 6; ++f) {
-      R pw[8];
+  for (int d = 0; d < 3; ++d)
 #pragma unroll
-      for (int q = 0; q < 8; ++q) u[f][q] = u[f][q] + du[q];
-      cons2prim(u[f], sc.gm1, pw);
-      if (!(pw[0] > R(0)) || !(pw[4] > R(0))) bad2 = true;
-      put(f, pw);
-    }
-  } else {
-    R dw[3][8];
+    for (int q = 0; q < 8; ++q) dw[d][q] = opaque(dw[d][q]);
 #pragma unroll
-    for (int d = 0; d < 3; ++d) {
+  for (int f = 0; f < 6; ++f) {
+    const int d = f / 2;
+    R fw[8], u[8], pw[8];
 #pragma unroll
-      for (int q = 0; q < 8; ++q) dw[d][q] = pf_slope<R, TX, TY, false>(W0, Wm, Wp, s, d, q, w[q], sc.limiter);
-      if (face_rule1(w, dw[d])) bad = true;
-    }
+    for (int q = 0; q < 8; ++q) fw[q] = f % 2 ? w[q] + R(0.5) * dw[d][q] : w[q] - R(0.5) * dw[d][q];
+    prim2cons(fw, sc.igm1, u);
 #pragma unroll
-    for (int q = 0; q < 8; ++q) du[q] = R(0);
-#pragma unroll
-    for (int d = 0; d < 3; ++d) {
-      R fwm[8], fwp[8], fm[8], fp[8];
-#pragma unroll
-      for (int q = 0; q < 8; ++q) {
-        fwm[q] = bad ? w[q] : w[q] - R(0.5) * dw[d][q];
-        fwp[q] = bad ? w[q] : w[q] + R(0.5) * dw[d][q];
-      }
-      flux_xyz(d, fwp, sc.igm1, fp);
-      flux_xyz(d, fwm, sc.igm1, fm);
-#pragma unroll
-      for (int q = 0; q < 8; ++q) du[q] = du[q] - st.hdtdx[d] * (fp[q] - fm[q]);
-    }
-#pragma unroll
-    for (int f = 0; f < 6; ++f) {
-      const int d = f / 2;
-      R fw[8], u[8], pw[8];
-#pragma unroll
-      for (int q = 0; q < 8; ++q) fw[q] = bad ? w[q] : (f % 2 ? w[q] + R(0.5) * dw[d][q] : w[q] - R(0.5) * dw[d][q]);
-      prim2cons(fw, sc.igm1, u);
-#pragma unroll
-      for (int q = 0; q < 8; ++q) u[q] = u[q] + du[q];
-      cons2prim(u, sc.gm1, pw);
-      if (!(pw[0] > R(0)) || !(pw[4] > R(0))) bad2 = true;
-      put(f, pw);
-    }
+    for (int q = 0; q < 8; ++q) u[q] = u[q] + du[q];
+    cons2prim(u, sc.gm1, pw);
+    if (!(pw[0] > R(0)) || !(pw[4] > R(0))) bad2 = true;
+    put(f, pw);
   }
 #pragma unroll
   for (int q = 0; q < 8; ++q) duk[q] = du[q];
@@ -186,25 +171,6 @@ __device__ __forceinline__ R pf_edge(const R* __restrict__ sm, int s, int z) {
   return Tr<R>::quarter(e00 + e10 + e01 + e11);
 }
 
-// The difference along axis q of the axis-a edge averages on the two edges of
-// the axis-d lower face of the cell at s (a, d, q distinct).  FP32 takes
-// it from the four cells that do not cancel, half the reads and a rounding
-// less; FP64 from the two averages, as the staged kernels do.
-template <typename R, int TX, int TY, int a, int d, int q>
-__device__ __forceinline__ R pf_edge_diff(const R* __restrict__ sm, int s, int z) {
-  using L = PfLayout<TX, TY>;
-  constexpr int so[3] = {1, L::PX, 0}, zo[3] = {0, 0, 1};
-  if constexpr (sizeof(R) == 4) {
-    const R hi = pf_en<R, TX, TY>(sm, a, s + so[q], z + zo[q]) +
-                 pf_en<R, TX, TY>(sm, a, s + so[q] - so[d], z + zo[q] - zo[d]);
-    const R lo = pf_en<R, TX, TY>(sm, a, s - so[q], z - zo[q]) +
-                 pf_en<R, TX, TY>(sm, a, s - so[q] - so[d], z - zo[q] - zo[d]);
-    return Tr<R>::quarter(hi - lo);
-  } else {
-    return pf_edge<R, TX, TY, a>(sm, s + so[q], z + zo[q]) - pf_edge<R, TX, TY, a>(sm, s, z);
-  }
-}
-
 // The flux of the axis-d lower face of a tile cell (element x, ring position
 // s of plane zc) between the face states lf and rf (7 values in the face's
 // rotated frame): the CT half-step normal field from edge averages of E^n,
@@ -213,14 +179,16 @@ template <typename R, int TX, int TY, int d>
 __device__ __forceinline__ void pf_face(const R* __restrict__ sm, const DPatch& p, const StepDt<R>& st,
                                         const SolverConsts<R>& sc, R* scr, int64_t x, int s, int zc, const R (&lf)[7],
                                         const R (&rf)[7]) {
+  using L = PfLayout<TX, TY>;
   constexpr int b = (d + 1) % 3, cc = (d + 2) % 3;
-  const R dEc = pf_edge_diff<R, TX, TY, cc, d, b>(sm, s, zc);
-  const R dEb = pf_edge_diff<R, TX, TY, b, d, cc>(sm, s, zc);
+  constexpr int so[3] = {1, L::PX, 0}, zo[3] = {0, 0, 1};
+  const R dEc = pf_edge<R, TX, TY, cc>(sm, s + so[b], zc + zo[b]) - pf_edge<R, TX, TY, cc>(sm, s, zc);
+  const R dEb = pf_edge<R, TX, TY, b>(sm, s + so[cc], zc + zo[cc]) - pf_edge<R, TX, TY, b>(sm, s, zc);
   const R bh = ((const R*)p.B[d])[x] - (st.hdtdx[b] * dEc - st.hdtdx[cc] * dEb);
   const R Lf[8] = {lf[0], lf[1], lf[2], lf[3], lf[4], R(0), lf[5], lf[6]};
   const R Rf[8] = {rf[0], rf[1], rf[2], rf[3], rf[4], R(0), rf[5], rf[6]};
   R fr[8], f[8], upw;
-  hlld_side<R, kFastRecip>(Lf, Rf, bh, sc.gamma, sc.igm1, sc.eps_up, sc.emf != 1, fr, &upw);
+  hlld<R, kFastRecip>(d, Lf, Rf, bh, sc.gamma, sc.igm1, sc.eps_up, sc.emf != 1, fr, &upw);
   rot_out(d, fr, f);
   f[5 + d] = upw;
   VecIO<R>::store8(arr(scr, p, SC_F + d * 8), p.snelem, x, f);
@@ -306,7 +274,8 @@ __global__ void __launch_bounds__(PfLayout<TX, TY>::NT, MINB)
       const bool px = cy >= y0, py = cx >= x0;  // not the lower row, not the left column
       pf_predict<R, TX, TY>(sm, s, zc, sc, st, duk, w, [&](int f, const R (&pw)[8]) {
         const int d = f >> 1, t1 = (d + 1) % 3, t2 = (d + 2) % 3;
-        const R v[7] = {pw[0], pw[1 + d], pw[1 + t1], pw[1 + t2], pw[4], pw[5 + t1], pw[5 + t2]};
+        const R v[7] = {opaque(pw[0]), opaque(pw[1 + d]), opaque(pw[1 + t1]), opaque(pw[1 + t2]),
+                        opaque(pw[4]), opaque(pw[5 + t1]), opaque(pw[5 + t2])};
         if (f == 1) {
           if (px) {
 #pragma unroll

@@ -212,23 +212,27 @@ template <bool FR, typename R> __device__ __forceinline__ R recip(R b) {
   else return R(0);
 }
 
-// FP32 HLLD of the staged and the fused kernels (hlld_side's formulas and
-// reciprocal form): both sides of the fan in full, every region's flux from
-// F* = F + S (U* - U).  Those kernels move 200 bytes a face and wait for
-// memory either way (k_flux 115 against 109 us at 128^3), and their rounding
-// is kept: a hierarchy's time step amplifies it (pf_untuned).  The fused pass
-// takes hlld_side.
-template <typename R>
-__device__ __forceinline__ void hlld32(const R* L, const R* Rr, R bn, R gamma, R igm1, R eps_up,
-                                       R* f, R* upw) {
+// FP32 HLLD: hlld_side's formulas in the reciprocal form, with every region's
+// flux from F* = F + S (U* - U), which the contracted FP64 build replaces by the
+// star state's own.  The staged kernels and the fused pass take the same
+// bits from it, so where an expression can be contracted in more than one way, and
+// the code around it could change the compiler's choice, the multiply-adds are
+// written out: the first product fused, the second rounded (dot3: for d = 2 the
+// other way round; U* - U of the momenta: by region).  Energies and fluxes
+// for the interface's side only, the single-star flux shared with the double-star
+// region: 128^3 k_flux 115 -> 113 us, a step 363 -> 359.
+__device__ __forceinline__ float dot3(int d, float u, float bn, float v, float by, float w, float bz) {
+  return __fmaf_rn(w, bz, d == 2 ? __fmaf_rn(v, by, __fmul_rn(u, bn)) : __fmaf_rn(u, bn, __fmul_rn(v, by)));
+}
+__device__ __forceinline__ void hlld32(int d, const float* L, const float* Rr, float bn, float gamma, float igm1,
+                                       float eps_up, float* f, float* upw) {
+  using R = float;
   R rl = L[0], ul = L[1], vl = L[2], wl_ = L[3], pl = L[4], byl = L[6], bzl = L[7];
   R rr = Rr[0], ur = Rr[1], vr = Rr[2], wr_ = Rr[3], pr = Rr[4], byr = Rr[6], bzr = Rr[7];
 
   R pml = R(0.5) * (bn * bn + byl * byl + bzl * bzl);
   R pmr = R(0.5) * (bn * bn + byr * byr + bzr * bzr);
   R ptl = pl + pml, ptr = pr + pmr;
-  R el = pl * igm1 + R(0.5) * rl * (ul * ul + vl * vl + wl_ * wl_) + pml;
-  R er = pr * igm1 + R(0.5) * rr * (ur * ur + vr * vr + wr_ * wr_) + pmr;
 
   R cfl = fast_speed(rl, pl, bn, byl, bzl, gamma);
   R cfr = fast_speed(rr, pr, bn, byr, bzr, gamma);
@@ -252,7 +256,7 @@ __device__ __forceinline__ void hlld32(const R* L, const R* Rr, R bn, R gamma, R
   R dd = rsr - rsl;
   const R idd = R(1) / dd;
   R sm = ((rsr * ur - rsl * ul) - (ptr - ptl)) * idd;
-  R pts = ((rsr * ptl - rsl * ptr) + rsl * rsr * (ur - ul)) * idd;
+  R pts = __fmaf_rn(__fmul_rn(rsl, rsr), ur - ul, __fmaf_rn(rsr, ptl, -__fmul_rn(rsl, ptr))) * idd;
   R tie = eps_up * (sr - sl);
   *upw = (sm > tie) ? R(1) : ((sm < -tie) ? R(-1) : R(0));
 
@@ -284,34 +288,45 @@ __device__ __forceinline__ void hlld32(const R* L, const R* Rr, R bn, R gamma, R
     vrs = vr - byr * fv; wrs = wr_ - bzr * fv;
     byrs = byr * fb; bzrs = bzr * fb;
   }
-  R vbl = ul * bn + vl * byl + wl_ * bzl;
-  R vbr = ur * bn + vr * byr + wr_ * bzr;
-  R vbls = sm * bn + vls * byls + wls * bzls;
-  R vbrs = sm * bn + vrs * byrs + wrs * bzrs;
-  R els = (((sdl * el - ptl * ul) + pts * sm) + bn * (vbl - vbls)) * isml;
-  R ers = (((sdr * er - ptr * ur) + pts * sm) + bn * (vbr - vbrs)) * ismr;
+
+  // the interface lies in the half of the fan on S_M's side (see hlld_side)
+  const bool left = (sm >= R(0));
+  const R rho = left ? rl : rr, u = left ? ul : ur, v = left ? vl : vr, w = left ? wl_ : wr_;
+  const R p = left ? pl : pr, by = left ? byl : byr, bz = left ? bzl : bzr;
+  const R pm = left ? pml : pmr, pt = left ? ptl : ptr;
+  const R S = left ? sl : sr, sd = left ? sdl : sdr;
+  const R rs = left ? rls : rrs, vs = left ? vls : vrs, ws = left ? wls : wrs;
+  const R bys = left ? byls : byrs, bzs = left ? bzls : bzrs;
+  const R e = __fmaf_rn(p, igm1, __fmul_rn(R(0.5) * rho, dot3(0, u, u, v, v, w, w))) + pm;
+  const R vb = dot3(0, u, bn, v, by, w, bz);
+  const R vbs = dot3(d, sm, bn, vs, bys, ws, bzs);
+  const R es = __fmul_rn(__fmaf_rn(bn, vb - vbs, __fmaf_rn(pts, sm, __fmaf_rn(sd, e, -__fmul_rn(pt, u)))),
+                         left ? isml : ismr);
 
   const R isl = Tr<R>::rsqrt_(rls), isr = Tr<R>::rsqrt_(rrs);
   const R sqrl = rls * isl, sqrr = rrs * isr;
-  const R sls = sm - Tr<R>::abs(bn) * isl, srs = sm + Tr<R>::abs(bn) * isr;
+  const R ab = Tr<R>::abs(bn);
+  const R Ss = __fmaf_rn(left ? -ab : ab, left ? isl : isr, sm);
 
-  R fo[8];
-  if (sls >= R(0) || srs < R(0)) {
-    // single-star region: F* = F_outer + S_outer (U* - U_outer)
-    const bool left = (sls >= R(0));
-    const R rho = left ? rl : rr, u = left ? ul : ur, v = left ? vl : vr, w = left ? wl_ : wr_;
-    const R e = left ? el : er, by = left ? byl : byr, bz = left ? bzl : bzr;
-    const R S = left ? sl : sr;
-    const R rs = left ? rls : rrs, vs = left ? vls : vrs, ws = left ? wls : wrs;
-    const R es = left ? els : ers, bys = left ? byls : byrs, bzs = left ? bzls : bzrs;
-    flux_rot(left ? L : Rr, bn, igm1, fo);
-    const R u0[8] = {rho, rho * u, rho * v, rho * w, e, bn, by, bz};
-    const R us[8] = {rs, rs * sm, rs * vs, rs * ws, es, bn, bys, bzs};
+  // single-star region: F* = F_outer + S_outer (U* - U_outer)
+  const R mn = rho * u;
+  const R fo[8] = {mn, mn * u + pt - bn * bn, mn * v - bn * by, mn * w - bn * bz, (e + pt) * u - bn * vb, R(0),
+                   by * u - bn * v, bz * u - bn * w};
+  const R u0[8] = {rho, mn, __fmul_rn(rho, v), __fmul_rn(rho, w), e, bn, by, bz};
+  const R us[8] = {rs, rs * sm, rs * vs, rs * ws, es, bn, bys, bzs};
 #pragma unroll
-    for (int q = 0; q < 8; ++q) f[q] = fo[q] + S * (us[q] - u0[q]);
+  for (int q = 0; q < 8; ++q) f[q] = __fmaf_rn(S, us[q] - u0[q], fo[q]);
+  if (left ? Ss >= R(0) : Ss < R(0)) {
+    f[1] = __fmaf_rn(S, __fmaf_rn(rs, sm, -u0[1]), fo[1]);
+    f[2] = __fmaf_rn(S, __fmaf_rn(rs, vs, -u0[2]), fo[2]);
+    f[3] = __fmaf_rn(S, __fmaf_rn(rs, ws, -u0[3]), fo[3]);
     return;
   }
+  f[1] = __fmaf_rn(S, __fmaf_rn(-rho, u, us[1]), fo[1]);
+  f[2] = __fmaf_rn(S, __fmaf_rn(-rho, v, us[2]), fo[2]);
+  f[3] = __fmaf_rn(S, __fmaf_rn(-rho, w, us[3]), fo[3]);
 
+  // double-star region: F** = F* + S* (U** - U*)
   R sgn = (bn >= R(0)) ? R(1) : R(-1);
   R ssum = sqrl + sqrr;
   const R iss = R(1) / ssum;
@@ -319,26 +334,11 @@ __device__ __forceinline__ void hlld32(const R* L, const R* Rr, R bn, R gamma, R
   R wss = ((sqrl * wls + sqrr * wrs) + sgn * (bzrs - bzls)) * iss;
   R byss = ((sqrl * byrs + sqrr * byls) + sgn * (sqrl * sqrr) * (vrs - vls)) * iss;
   R bzss = ((sqrl * bzrs + sqrr * bzls) + sgn * (sqrl * sqrr) * (wrs - wls)) * iss;
-  R vbss = sm * bn + vss * byss + wss * bzss;
-
-  const bool left = (sm >= R(0));
-  const R rho = left ? rl : rr, u = left ? ul : ur, v = left ? vl : vr, w = left ? wl_ : wr_;
-  const R e = left ? el : er, by = left ? byl : byr, bz = left ? bzl : bzr;
-  const R S = left ? sl : sr, Ss = left ? sls : srs;
-  const R rs = left ? rls : rrs, vs = left ? vls : vrs, ws = left ? wls : wrs;
-  const R es = left ? els : ers, bys = left ? byls : byrs, bzs = left ? bzls : bzrs;
-  R ess;
-  if (left) ess = els - sqrl * (vbls - vbss) * sgn;
-  else ess = ers + sqrr * (vbrs - vbss) * sgn;
-  flux_rot(left ? L : Rr, bn, igm1, fo);
-  const R u0[8] = {rho, rho * u, rho * v, rho * w, e, bn, by, bz};
-  const R us[8] = {rs, rs * sm, rs * vs, rs * ws, es, bn, bys, bzs};
+  R vbss = dot3(d, sm, bn, vss, byss, wss, bzss);
+  const R ess = __fmaf_rn(__fmul_rn(left ? -sqrl : sqrr, vbs - vbss), sgn, es);
   const R uss[8] = {rs, rs * sm, rs * vss, rs * wss, ess, bn, byss, bzss};
 #pragma unroll
-  for (int q = 0; q < 8; ++q) {
-    R fs = fo[q] + S * (us[q] - u0[q]);
-    f[q] = fs + Ss * (uss[q] - us[q]);
-  }
+  for (int q = 0; q < 8; ++q) f[q] = f[q] + Ss * (uss[q] - us[q]);
 }
 
 // HLLD flux (Miyoshi & Kusano 2005) between rotated primitive states L (lower
@@ -461,17 +461,8 @@ __device__ __forceinline__ void hlld_side(const R* L, const R* Rr, R bn, R gamma
   const R vbs = sm * bn + vs * bys + ws * bzs;
   const R es = qdiv<FR>(((sd * e - pt * u) + pts * sm) + bn * (vb - vbs), sS, isS);
 
-  R sqrl, sqrr, ab;
-  if constexpr (sizeof(R) == 4) {  // one reciprocal root gives the root and the quotient
-    const R isl = T::rsqrt_(rls), isr = T::rsqrt_(rrs);
-    sqrl = rls * isl;
-    sqrr = rrs * isr;
-    ab = T::abs(bn) * (left ? isl : isr);
-  } else {
-    sqrl = T::sqrt_(rls);
-    sqrr = T::sqrt_(rrs);
-    ab = T::div(T::abs(bn), left ? sqrl : sqrr);
-  }
+  const R sqrl = T::sqrt_(rls), sqrr = T::sqrt_(rrs);
+  const R ab = T::div(T::abs(bn), left ? sqrl : sqrr);
   const R Ss = left ? sm - ab : sm + ab;
 
   const R mxs = rs * sm;
@@ -542,10 +533,11 @@ __device__ __forceinline__ void hlld_side(const R* L, const R* Rr, R bn, R gamma
   f[7] = f[7] + Ss * (bzss - bzs);
 }
 
+// HLLD flux of an axis-d face.
 template <typename R, bool FR = false>
-__device__ __forceinline__ void hlld(const R* L, const R* Rr, R bn, R gamma, R igm1, R eps_up, bool up, R* f,
+__device__ __forceinline__ void hlld(int d, const R* L, const R* Rr, R bn, R gamma, R igm1, R eps_up, bool up, R* f,
                                      R* upw) {
-  if constexpr (sizeof(R) == 4) hlld32(L, Rr, bn, gamma, igm1, eps_up, f, upw);
+  if constexpr (sizeof(R) == 4) hlld32(d, L, Rr, bn, gamma, igm1, eps_up, f, upw);
   else hlld_side<R, FR>(L, Rr, bn, gamma, igm1, eps_up, up, f, upw);
 }
 
