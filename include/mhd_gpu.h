@@ -98,7 +98,8 @@ typedef struct {
   int32_t advance_kernel; /* 0: the context's choice (what mhd_autotune_advance
                         measured fastest; before that the fused pass for
                         MHD_F32 calls of mhd_patch_advance without captures
-                        and grown boxes, else the staged kernels);
+                        and grown boxes from 2^18 cells on, two layers around
+                        each patch counted, else the staged kernels);
                         1: the staged kernels (one launch per stage,
                         intermediates in the scratch arena; the predictor
                         tiled in shared memory if the autotuner chose it);

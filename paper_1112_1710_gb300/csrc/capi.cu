@@ -628,24 +628,33 @@ int64_t pf_tiles(const PatchSize& q, int tx, int ty) {
 
 // Is an advance that nobody tuned or forced run by the fused pass?  (Either way
 // the same bits.)  FP64 is bound by its own pipe in both and stays staged.
-// FP32 patches advanced with a given dt (serving batches) take it: staged against fused
-// pass 41 / 41 us for a batch of 131 k cells, 134 / 119 for 524 k, 841 / 771 for
-// 4.2 M.  Steps that reduce their own CFL dt and calls of a hierarchy
-// (flux-register captures, grown update boxes) stay staged unless tuned.
+// FP32 patches advanced with a given dt (serving batches) take it where they fill
+// the GPU: from 2^18 cells on, the patches grown by the two layers the staged
+// stages compute.  Staged against fused pass, us with the upwinded EMF (grown
+// cells): one cube of 32^3 (47 k) 26.7 / 28.7, 48^3 (141 k) 36.9 / 36.9, 64^3
+// (314 k) 72.2 / 63.7; batches of 16 x 16^3 (128 k) 32.8 / 48.3, 4 x 32^3 (187 k)
+// 46.6 / 47.2, 2 x 48^3 (281 k) 66.7 / 59.5, 256 x 8^3 (442 k) 105 / 72, 32 x
+// 24^3 (702 k, items that fill the last round badly) 156 / 174, mixed 4.2 M cells
+// 841 / 771; one plane of 128^2 (87 k) 28.8 / 27.0, 256^2 (338 k) 49.2 / 36.9.
+// Steps that reduce their own CFL dt and calls of a hierarchy (flux-register
+// captures, grown update boxes) stay staged unless tuned.
 bool pf_untuned(const std::vector<PatchSize>& ps, int dtype, int32_t ncap, bool cfl_dt) {
   if (dtype != MHD_F32 || ncap > 0 || cfl_dt) return false;
-  for (const PatchSize& q : ps)
+  int64_t cells = 0;
+  for (const PatchSize& q : ps) {
     if (q.k > 0) return false;
-  return true;
+    cells += (int64_t)(q.n[0] + 4) * (q.n[1] + 4) * (q.n[2] + 4);
+  }
+  return cells >= 1 << 18;
 }
 
 // Planes per work item of the fused pass.  The blocks of a call run in rounds
 // of `slots`; a round costs an item's planes and kPfStart planes for its start.
 // The length with the shortest rounds, taking a last round that is part full at
 // half way between its share and a whole one (it runs with less company on its
-// SMs).  128^3 in FP32 (81 tiles of 130 planes, 304 slots): 4 planes 377 us a step,
-// 8 362, 12 348, 16 388, 24 383, 33 451; the rule takes 12.  Hundreds of small
-// patches fill many rounds, and whole columns win.
+// SMs).  128^3 in FP32 (81 tiles of 130 planes, 304 slots): 4 planes 388 us a step,
+// 8 372, 12 361, 16 393, 24 389, 33 455, 44 398; the rule takes 40 (386).  Hundreds
+// of small patches fill many rounds, and whole columns win.
 int pf_chunk(const std::vector<PatchSize>& ps, int tx, int ty, int slots) {
   constexpr double kPfStart = 1.6;
   int zmax = 1;

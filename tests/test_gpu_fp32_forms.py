@@ -124,3 +124,25 @@ def test_hierarchy_fp32_per_patch_equals_batched(capi, kind):
         for h in hs:
             h.close()
         capi.mhd_ctx_destroy(ctx)
+
+
+@pytest.mark.parametrize("sizes,fused", [([(220, 220, 1)], False), ([(230, 230, 1)], True), ([(59, 60, 60)], False),
+                                         ([(60, 60, 60)], True), ([(8, 8, 8)] * 151, False), ([(8, 8, 8)] * 152, True)])
+def test_untuned_route_by_size(capi, sizes, fused):
+    """Kernel launches of an untuned call on both sides of 2^18 grown cells
+    (arithmetic-mean EMF: five staged, three with the fused pass), and the bits of
+    the staged kernels either way."""
+    out = []
+    for kernel in (0, 1):
+        ctx = capi.mhd_ctx_create(emf=1, advance_kernel=kernel)
+        ps = [to_patch(_moving(n, 2, 5, 0.5), n, 2, DX, dtype="f32", pid=i) for i, n in enumerate(sizes)]
+        d = torch.full((1,), 1e-3, dtype=torch.float64, device="cuda")
+        try:
+            before = capi.mhd_launch_count(ctx)
+            capi.mhd_patch_advance(ctx, [p.desc() for p in ps], d.data_ptr())
+            assert capi.mhd_launch_count(ctx) - before == (3 if fused and kernel == 0 else 5)
+            out.append([p.state.cpu().numpy() for p in ps])
+        finally:
+            capi.mhd_ctx_destroy(ctx)
+    for a, b in zip(*out):
+        assert np.array_equal(a, b)
