@@ -233,6 +233,14 @@ MHD_HD bool abs_gt(double x, double t) {
 MHD_HD bool less_mag(double a, double b) {
   return (bits(a) & 0x7fffffffffffffffull) < (bits(b) & 0x7fffffffffffffffull);
 }
+MHD_HD bool nan(double x) { return (bits(x) & 0x7fffffffffffffffull) > 0x7ff0000000000000ull; }
+// any of the three an infinity or NaN?  (their upper words' exponents)
+MHD_HD bool any_special(double a, double b, double c) {
+  const uint32_t x = (uint32_t)(bits(a) >> 32) << 1, y = (uint32_t)(bits(b) >> 32) << 1, z = (uint32_t)(bits(c) >> 32) << 1;
+  const uint32_t m = x > y ? x : y;
+  return (m > z ? m : z) >= 0xffe00000u;
+}
+MHD_HD bool special(double a) { return (uint32_t)(bits(a) >> 32) << 1 >= 0xffe00000u; }
 // Is |d| > 1e-12 max(a1 a2, b) plain from the exponents (b finite)?
 MHD_HD bool clearly_above(double d, double a1, double a2, double b) {
   const int ed = (int)(bits(d) >> 52) & 0x7ff, e1 = (int)(bits(a1) >> 52) & 0x7ff,

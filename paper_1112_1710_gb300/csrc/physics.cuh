@@ -42,6 +42,10 @@ template <> struct Tr<double> {
   __device__ static __forceinline__ bool ge0(double x) { return i64::ge0(x); }
   __device__ static __forceinline__ bool abs_gt(double x, double t) { return i64::abs_gt(x, t); }
   __device__ static __forceinline__ bool less_mag(double a, double b) { return i64::less_mag(a, b); }
+  __device__ static __forceinline__ bool nan(double x) { return i64::nan(x); }
+  __device__ static __forceinline__ bool special(double x) { return i64::special(x); }
+  __device__ static __forceinline__ bool any_special(double a, double b, double c) { return i64::any_special(a, b, c); }
+  __device__ static __forceinline__ double undef() { return i64::value(0x7ff8000000000000ull); }
   __device__ static __forceinline__ double degen() { return 1e-12; }
   // |den| <= degen max(a1 a2, b); the exponents settle it almost always
   __device__ static __forceinline__ bool degenerate(double den, double a1, double a2, double b) {
@@ -60,13 +64,8 @@ template <> struct Tr<float> {
   __device__ static __forceinline__ float times4(float x) { return 4.0f * x; }
   __device__ static __forceinline__ bool pos(float x) { return x > 0.0f; }
   __device__ static __forceinline__ bool neg(float x) { return x < 0.0f; }
-  __device__ static __forceinline__ bool ge0(float x) { return x >= 0.0f; }
-  __device__ static __forceinline__ bool abs_gt(float x, float t) { return fabsf(x) > t; }
   __device__ static __forceinline__ bool less_mag(float a, float b) { return fabsf(a) < fabsf(b); }
   __device__ static __forceinline__ float degen() { return 1e-5f; }
-  __device__ static __forceinline__ bool degenerate(float den, float a1, float a2, float b) {
-    return fabsf(den) <= degen() * fmaxf(a1 * a2, b);
-  }
 };
 template <typename R> __device__ __forceinline__ R flip(R x, bool c) { return c ? -x : x; }
 
@@ -373,10 +372,16 @@ __device__ __forceinline__ void hlld_side(const R* L, const R* Rr, R bn, R gamma
 
   R cfl = fast_speed(rl, pl, bn, byl, bzl, gamma);
   R cfr = fast_speed(rr, pr, bn, byr, bzr, gamma);
-  R cmax = T::less_mag(cfr, cfl) ? cfl : cfr;
+  // max(cfl, cfr), min(ul, ur) and max(ul, ur), as a > b ? a : b and a < b ? a : b
+  // (a NaN in a gives b)
   const bool ulo = ul < ur;
+  R cmax = T::less_mag(cfr, cfl) ? cfl : cfr, umax = ulo ? ur : ul;
+  if (T::any_special(cfl, ul, ur)) {
+    if (T::nan(cfl)) cmax = cfr;
+    if (T::nan(ul) || T::nan(ur)) umax = ur;
+  }
   R sl = (ulo ? ul : ur) - cmax;
-  R sr = (ulo ? ur : ul) + cmax;
+  R sr = umax + cmax;
 
   if (T::ge0(sl)) {
     flux_rot(L, bn, igm1, f);
@@ -502,6 +507,10 @@ __device__ __forceinline__ void hlld_side(const R* L, const R* Rr, R bn, R gamma
       f[6] = f[6] + bys * (u - sm);
       f[7] = f[7] + bzs * (u - sm);
     }
+    if (!single && T::special(Ss)) {  // (a state with rho <= 0)
+#pragma unroll
+      for (int q = 0; q < 8; ++q) f[q] = T::undef();
+    }
     return;
   }
   // outer flux and conserved states; single-star region: F* = F + S (U* - U)
@@ -517,7 +526,12 @@ __device__ __forceinline__ void hlld_side(const R* L, const R* Rr, R bn, R gamma
   f[7] = (bz * u - bn * w) + S * (bzs - bz);
   if (single) return;
 
-  // double-star region: F** = F* + S* (U** - U*); rho and S_M are U*'s
+  // double-star region: F** = F* + S* (U** - U*); rho and S_M are U*'s, whose
+  // zero jumps still carry what is not finite
+  if (T::any_special(Ss, rs, mxs)) {
+    if (T::special(Ss) || T::special(rs)) f[0] = T::undef();
+    if (T::special(Ss) || T::special(mxs)) f[1] = T::undef();
+  }
   R ssum = sqrl + sqrr;
   R vss = T::div((sqrl * vls + sqrr * vrs) + flip(byrs - byls, bneg), ssum);
   R wss = T::div((sqrl * wls + sqrr * wrs) + flip(bzrs - bzls, bneg), ssum);
