@@ -39,6 +39,8 @@
  * cached by content, so after one warm-up call with the same arguments a call
  * uploads nothing and can be captured in a CUDA graph; a captured graph holds
  * the scratch address, which changes only when a larger call grows the arena.
+ * The tables a captured call read stay until the context is destroyed; of the
+ * others some 256 MB are kept.
  */
 #ifndef MHD_GPU_H
 #define MHD_GPU_H

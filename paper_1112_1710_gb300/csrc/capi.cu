@@ -34,6 +34,8 @@ struct TableEntry {
   int kind = 0;       // what the key describes (TableKind)
   void* dev = nullptr;
   size_t count = 0;   // elements of the table
+  size_t bytes = 0;   // its size with the key's
+  bool pinned = false;  // used by a call under capture: the graph reads it at every replay
 };
 
 enum TableKind : int {
@@ -86,7 +88,8 @@ struct mhd_ctx {
   size_t rflags_bytes = 0;
   std::string err;
   std::unordered_multimap<uint64_t, TableEntry> tables;
-  size_t table_bytes = 0;
+  size_t table_bytes = 0, pinned_bytes = 0;
+  bool capturing = false;  // the current call's stream
   int64_t launches = 0;
   // advance path per element type (index MHD_F64 / MHD_F32) as picked by the
   // autotuner: staged or fused, the fused variant and its z-chunk length (0:
@@ -135,8 +138,12 @@ mhd_status keyed_table(mhd_ctx* c, int kind, const void* key, size_t nkey, Build
   const uint64_t h = hash_bytes(kind, key, nkey);
   auto range = c->tables.equal_range(h);
   for (auto it = range.first; it != range.second; ++it) {
-    const TableEntry& e = it->second;
+    TableEntry& e = it->second;
     if (e.kind == kind && e.key.size() == nkey && (nkey == 0 || std::memcmp(e.key.data(), key, nkey) == 0)) {
+      if (c->capturing && !e.pinned) {
+        e.pinned = true;
+        c->pinned_bytes += e.bytes;
+      }
       *out = (const T*)e.dev;
       *count = (int)e.count;
       return MHD_OK;
@@ -162,7 +169,10 @@ mhd_status keyed_table(mhd_ctx* c, int kind, const void* key, size_t nkey, Build
   }
   *out = (const T*)t.dev;
   *count = (int)t.count;
-  c->table_bytes += n + nkey;
+  t.bytes = n + nkey;
+  t.pinned = c->capturing;
+  c->table_bytes += t.bytes;
+  if (t.pinned) c->pinned_bytes += t.bytes;
   c->tables.emplace(h, std::move(t));
   return MHD_OK;
 }
@@ -266,15 +276,34 @@ mhd_status begin(mhd_ctx* c) {
   if (!c) return MHD_EINVAL;
   cudaError_t e = cudaSetDevice(c->device);
   if (e != cudaSuccess) return cuda_fail(c, e, "cudaSetDevice");
-  if (c->table_bytes > kTableCacheLimit) {
-    // drop every cached table, between calls (a call's own tables stay);
+  return MHD_OK;
+}
+
+// Start of a call that enqueues on `stream`.  Past the cache's limit every table
+// is dropped but those that a captured graph reads; never under capture, which
+// must not synchronise, and between calls only (a call's own tables stay).
+mhd_status begin(mhd_ctx* c, void* stream) {
+  mhd_status r = begin(c);
+  if (r) return r;
+  cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing((cudaStream_t)stream, &cs) != cudaSuccess) {
+    cudaGetLastError();  // the legacy stream while another one is captured
+    cs = cudaStreamCaptureStatusActive;
+  }
+  c->capturing = cs != cudaStreamCaptureStatusNone;
+  if (!c->capturing && c->table_bytes - c->pinned_bytes > kTableCacheLimit) {
     // launches in flight may still read them
-    e = cudaDeviceSynchronize();
+    cudaError_t e = cudaDeviceSynchronize();
     if (e != cudaSuccess) return cuda_fail(c, e, "table cache flush");
-    for (auto& kv : c->tables)
-      if (kv.second.dev) cudaFree(kv.second.dev);
-    c->tables.clear();
-    c->table_bytes = 0;
+    for (auto it = c->tables.begin(); it != c->tables.end();) {
+      if (it->second.pinned) {
+        ++it;
+        continue;
+      }
+      if (it->second.dev) cudaFree(it->second.dev);
+      it = c->tables.erase(it);
+    }
+    c->table_bytes = c->pinned_bytes;
   }
   return MHD_OK;
 }
@@ -847,7 +876,7 @@ static mhd_status scan_captures(mhd_ctx* c, std::vector<DPatch>& dp, const mhd_c
 static mhd_status advance_impl(mhd_ctx* c, const mhd_patch_desc* patches, int32_t n, const int32_t* grow,
                         const double* d_dt, const double* dt_scale, const mhd_capture* caps, int32_t ncap,
                         void* stream, bool cfl_dt) {
-  mhd_status r = begin(c);
+  mhd_status r = begin(c, stream);
   if (r) return r;
   if (n < 0 || (n > 0 && !patches)) return fail(c, MHD_EINVAL, "bad patch array");
   if (!d_dt) return fail(c, MHD_EINVAL, "d_dt is NULL");
@@ -966,7 +995,7 @@ mhd_status mhd_patch_step_cfl(mhd_ctx* c, const mhd_patch_desc* patches, int32_t
 mhd_status mhd_autotune_advance(mhd_ctx* c, const mhd_patch_desc* patches, int32_t n, const int32_t* grow,
                                 const mhd_capture* caps, int32_t ncap, const double* d_dt, int32_t reps,
                                 int32_t* variant_out, int32_t* chunk_out, float* ms_out, void* stream) {
-  mhd_status r = begin(c);
+  mhd_status r = begin(c, stream);
   if (r) return r;
   if (n < 1 || !patches || !d_dt || reps < 1 || reps > 1000) return fail(c, MHD_EINVAL, "autotune: bad arguments");
   if (ncap < 0 || (ncap > 0 && !caps)) return fail(c, MHD_EINVAL, "bad capture list");
@@ -1135,7 +1164,7 @@ mhd_status mhd_autotune_advance(mhd_ctx* c, const mhd_patch_desc* patches, int32
 
 mhd_status mhd_cfl_dt(mhd_ctx* c, const mhd_patch_desc* patches, int32_t n, const double* scale,
                       double* d_dt_out, void* stream) {
-  mhd_status r = begin(c);
+  mhd_status r = begin(c, stream);
   if (r) return r;
   if (n < 1 || !patches) return fail(c, MHD_EINVAL, "cfl_dt needs at least one patch");
   if (!d_dt_out) return fail(c, MHD_EINVAL, "d_dt_out is NULL");
@@ -1164,7 +1193,7 @@ mhd_status mhd_cfl_dt(mhd_ctx* c, const mhd_patch_desc* patches, int32_t n, cons
 
 mhd_status mhd_transfer_copy(mhd_ctx* c, const mhd_patch_desc* old, int32_t no, const mhd_patch_desc* fresh,
                              int32_t nn, const mhd_transfer_item* items, int32_t ni, void* stream) {
-  mhd_status r = begin(c);
+  mhd_status r = begin(c, stream);
   if (r) return r;
   if (no < 1 || nn < 1 || !old || !fresh || ni < 0 || (ni > 0 && !items))
     return fail(c, MHD_EINVAL, "transfer_copy: bad arguments");
@@ -1220,7 +1249,7 @@ mhd_status mhd_transfer_copy(mhd_ctx* c, const mhd_patch_desc* old, int32_t no, 
 mhd_status mhd_prolong_new(mhd_ctx* c, const mhd_patch_desc* coarse, int32_t nc, const mhd_patch_desc* fine,
                            int32_t nf, const mhd_prolong_new_item* items, int32_t ni, int32_t energy_mode,
                            unsigned long long* d_fallbacks, void* stream) {
-  mhd_status r = begin(c);
+  mhd_status r = begin(c, stream);
   if (r) return r;
   if (nc < 1 || nf < 1 || !coarse || !fine || ni < 0 || (ni > 0 && !items) || (energy_mode != 0 && energy_mode != 1))
     return fail(c, MHD_EINVAL, "prolong_new: bad arguments");
@@ -1288,7 +1317,7 @@ mhd_status mhd_prolong_new(mhd_ctx* c, const mhd_patch_desc* coarse, int32_t nc,
 }
 
 mhd_status mhd_floor(mhd_ctx* c, const mhd_patch_desc* patches, int32_t n, void* stream) {
-  mhd_status r = begin(c);
+  mhd_status r = begin(c, stream);
   if (r) return r;
   if (n < 1 || !patches) return fail(c, MHD_EINVAL, "floor: bad arguments");
   if (!(c->prm.p_floor > 0.0 || c->prm.rho_floor > 0.0)) return MHD_OK;
@@ -1361,7 +1390,7 @@ static void flag_tiles(const std::vector<PatchSize>& ps, std::vector<FusedItem>&
 
 mhd_status mhd_flag_cells(mhd_ctx* c, const mhd_patch_desc* patches, int32_t n, double theta, uint8_t* d_flags,
                           void* stream) {
-  mhd_status r = begin(c);
+  mhd_status r = begin(c, stream);
   if (r) return r;
   if (n < 1 || !patches || !d_flags || !(theta >= 0.0)) return fail(c, MHD_EINVAL, "flag_cells: bad arguments");
   std::vector<DPatch> dp(n);
@@ -1442,7 +1471,7 @@ static void ghost_tasks(const std::vector<DCopy>& dc, int dtype, std::vector<Gho
 
 mhd_status mhd_ghost_fill(mhd_ctx* c, const mhd_patch_desc* patches, int32_t n, const mhd_copy* list,
                           int32_t nlist, void* stream) {
-  mhd_status r = begin(c);
+  mhd_status r = begin(c, stream);
   if (r) return r;
   if (n < 0 || (n > 0 && !patches) || nlist < 0 || (nlist > 0 && !list))
     return fail(c, MHD_EINVAL, "bad arguments");
@@ -1511,7 +1540,7 @@ mhd_status mhd_ghost_fill(mhd_ctx* c, const mhd_patch_desc* patches, int32_t n, 
 
 mhd_status mhd_conservation_sums(mhd_ctx* c, const mhd_patch_desc* patches, int32_t n, double* d_out8,
                                  void* stream) {
-  mhd_status r = begin(c);
+  mhd_status r = begin(c, stream);
   if (r) return r;
   if (n < 1 || !patches || !d_out8) return fail(c, MHD_EINVAL, "bad arguments");
   std::vector<DPatch> dp(n);
@@ -1537,7 +1566,7 @@ mhd_status mhd_conservation_sums(mhd_ctx* c, const mhd_patch_desc* patches, int3
 
 mhd_status mhd_prolong(mhd_ctx* c, const mhd_patch_desc* coarse, int32_t nc, const mhd_patch_desc* fine,
                        int32_t nf, const mhd_prolong_item* items, int32_t n, void* stream) {
-  mhd_status r = begin(c);
+  mhd_status r = begin(c, stream);
   if (r) return r;
   if (n < 0 || (n > 0 && !items)) return fail(c, MHD_EINVAL, "bad item list");
   if (n == 0) return MHD_OK;
@@ -1585,7 +1614,7 @@ mhd_status mhd_prolong(mhd_ctx* c, const mhd_patch_desc* coarse, int32_t nc, con
 
 mhd_status mhd_restrict(mhd_ctx* c, const mhd_patch_desc* fine, int32_t nf, const mhd_patch_desc* coarse,
                         int32_t nc, const mhd_restrict_item* items, int32_t n, void* stream) {
-  mhd_status r = begin(c);
+  mhd_status r = begin(c, stream);
   if (r) return r;
   if (n < 0 || (n > 0 && !items)) return fail(c, MHD_EINVAL, "bad item list");
   if (n == 0) return MHD_OK;
@@ -1637,7 +1666,7 @@ mhd_status mhd_restrict(mhd_ctx* c, const mhd_patch_desc* fine, int32_t nf, cons
 mhd_status mhd_restrict_prolong(mhd_ctx* c, int32_t mode, const mhd_patch_desc* fine, int32_t nf,
                                 const mhd_patch_desc* coarse, int32_t nc, const mhd_level_item* items, int32_t n,
                                 void* stream) {
-  mhd_status r = begin(c);
+  mhd_status r = begin(c, stream);
   if (r) return r;
   if (mode != MHD_PROLONG && mode != MHD_RESTRICT) return fail(c, MHD_EINVAL, "mode %d", mode);
   if (n < 0 || (n > 0 && !items)) return fail(c, MHD_EINVAL, "bad item list");
@@ -1661,7 +1690,7 @@ mhd_status mhd_restrict_prolong(mhd_ctx* c, int32_t mode, const mhd_patch_desc* 
 
 mhd_status mhd_reflux(mhd_ctx* c, const mhd_patch_desc* coarse, int32_t nc, double* const* corr,
                       const mhd_deposit* deps, int32_t nd, void* stream) {
-  mhd_status r = begin(c);
+  mhd_status r = begin(c, stream);
   if (r) return r;
   if (nc < 1 || !corr || nd < 0 || (nd > 0 && !deps)) return fail(c, MHD_EINVAL, "bad arguments");
   int dtype = -1;
