@@ -11,6 +11,7 @@ from __future__ import annotations
 
 import ctypes
 import itertools
+import operator
 import struct
 from dataclasses import dataclass
 
@@ -62,9 +63,13 @@ class Patch:
         sq, sz, sy, _ = st.stride()
         base, plane = st.data_ptr(), sq * st.element_size()
         # the fields in the order of mhd_patch_desc, packed in one call
-        return capi.mhd_patch_desc.from_buffer_copy(_DESC.pack(
-            self.level, self.g, self.dtype_code, self.patch_id, *map(int, self.lo), *map(int, self.hi),
-            *range(base, base + 8 * plane, plane), 1, sy, sz, *map(float, self.dx)))
+        ints = (self.level, self.g, self.dtype_code, self.patch_id, *map(int, self.lo), *map(int, self.hi))
+        rest = (*range(base, base + 8 * plane, plane), 1, sy, sz, *map(float, self.dx))
+        try:
+            raw = _DESC.pack(*ints, *rest)
+        except struct.error:  # beyond 32 bits: modulo 2^32, as ctypes assigns them
+            raw = _DESC.pack(*((operator.index(v) + 2 ** 31) % 2 ** 32 - 2 ** 31 for v in ints), *rest)
+        return capi.mhd_patch_desc.from_buffer_copy(raw)
 
     @staticmethod
     def from_array(arr, lo, n, g, dx, dtype="f64", device="cuda", level=0, patch_id=0) -> "Patch":
