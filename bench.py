@@ -71,6 +71,7 @@ def parse():
     ap.add_argument("--advance", default="auto", choices=list(ADVANCE_KERNELS),
                     help="advance of the single patch and of the hierarchies: the autotuner's choice, or forced "
                          "(staged kernels, fused pass, fused kernel)")
+    ap.add_argument("--full", action="store_true", help="print the whole record on stdout (default: on stderr)")
     ap.add_argument("--requests", type=int, default=10000, help="serve: requests per offered load")
     ap.add_argument("--slots", type=int, default=3, help="serve: streams (one context each)")
     ap.add_argument("--batch-cells", type=int, default=4 << 20, help="serve: cell budget of one batch")
@@ -82,6 +83,35 @@ def parse():
     ap.add_argument("--serve-requests", type=int, default=2000,
                     help="default run: requests per offered load of the serving config")
     return ap.parse_args()
+
+
+# entries printed whole; of the other nested ones the line carries the scalars
+WHOLE = ("config", "roofline", "hbm_step", "e2e", "clocks", "cpu_baseline")
+
+
+def short_line(line):
+    """The record without what is nested deeper than one level (readers of the
+    default run's stdout take a line of some 8 KB at most; the whole record has
+    25 KB)."""
+    out = {}
+    for k, v in line.items():
+        if k not in WHOLE and isinstance(v, dict):
+            v = {a: b for a, b in v.items() if not isinstance(b, (dict, list)) and len(str(b)) <= 60}
+        elif k not in WHOLE and isinstance(v, list):
+            continue
+        out[k] = v
+    return out
+
+
+def emit(line, to_stdout=False):
+    """The one JSON line on stdout; the whole record on stderr (with --full on
+    stdout instead)."""
+    full = json.dumps(line)
+    if to_stdout:
+        print(full)
+        return
+    print(full, file=sys.stderr, flush=True)
+    print(json.dumps(short_line(line)))
 
 
 def config(n):
@@ -543,7 +573,7 @@ def run_reference(args):
             "cpu_baseline": {"value": v, "unit": UNIT, "cores": cores, "kind": "oracle",
                              "sample": "%d full FP64 steps of the %d^3 blast on the host cores" % (args.steps, args.n)},
             "e2e": {"value": v, "unit": UNIT, "h2d_bytes_per_step": 0, "d2h_bytes_per_step": 0}}
-    print(json.dumps(line))
+    emit(line, args.full)
 
 
 def run_ours(args):
@@ -641,7 +671,7 @@ def run_ours(args):
         line["amr"] = measure_amr(args, local)
         torch.cuda.empty_cache()
         line["serving"] = measure_serve(args, local)
-    print(json.dumps(line))
+    emit(line, args.full)
 
 
 def amr_hierarchy(n0=64):
@@ -972,7 +1002,7 @@ def run_amr(args):
             "runs": res, "kernels_f32": attribution, "metadata": meta, "hilbert": hil, "regrid": rg}
     if cpu:
         line["cpu_baseline"] = cpu
-    print(json.dumps(line))
+    emit(line, args.full)
 
 
 def run_ot2d(args):
@@ -1040,7 +1070,7 @@ def run_ot2d(args):
         line["cpu_baseline"] = {"value": pr.cells * steps / dt, "unit": UNIT,
                                 "cores": O.get_threads(),
                                 "kind": "oracle", "sample": "the whole workload (100 steps), %.1f s" % dt}
-    print(json.dumps(line))
+    emit(line, args.full)
 
 
 def per_patch_f64(tpl, reqs, local, contract=0):
@@ -1151,7 +1181,7 @@ def run_serve(args):
             pr = synth.blast(r.n, g=G, seed=4242 + r.n)
             items.append((pr.state, pr.n, G, pr.dx, (0,), True))
         line["cpu_baseline"] = cpu_baseline_sample(items, "the first 400 requests of the same stream")
-    print(json.dumps(line))
+    emit(line, args.full)
 
 
 def run_deep(args):
@@ -1172,7 +1202,7 @@ def run_deep(args):
     line.update({"metric": METRIC, "n_gpus": world, "steps": args.deep_steps, "warmup": 2,
                  "ms_per_step": res["ms_per_coarse_step"], "higher_is_better": True, "scaling": "weak",
                  "vs_baseline": None, "data": "synthetic"})
-    print(json.dumps(line))
+    emit(line, args.full)
 
 
 def run_amr_step(args):
