@@ -1157,7 +1157,13 @@ mhd_status mhd_autotune_advance(mhd_ctx* c, const mhd_patch_desc* patches, int32
   c->pf_variant[di] = bv <= -3 ? -3 - bv : 0;
   c->fused_chunk[di] = bv >= 0 || bv <= -3 ? bcz : 0;
   if (variant_out) *variant_out = bv;
-  if (chunk_out) *chunk_out = bv <= -3 && bcz == 0 ? zmax + 2 : bcz;  // pf_chunk's choice at each call
+  if (chunk_out) {
+    *chunk_out = bcz;
+    if (bv <= -3 && bcz == 0) {  // each call's own choice: the one timed here
+      const PfVariant& pv = dtype == MHD_F32 ? kPfVariants32[-3 - bv] : kPfVariants64[-3 - bv];
+      *chunk_out = std::min(pf_chunk(ps, pv.tx, pv.ty, pv.minb * c->nsm), zmax + 2);
+    }
+  }
   if (ms_out) *ms_out = best;
   return MHD_OK;
 }

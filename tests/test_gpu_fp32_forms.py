@@ -146,3 +146,21 @@ def test_untuned_route_by_size(capi, sizes, fused):
             capi.mhd_ctx_destroy(ctx)
     for a, b in zip(*out):
         assert np.array_equal(a, b)
+
+
+@pytest.mark.parametrize("n", [(100, 40, 40), (31, 29, 102)])
+def test_autotune_reports_the_planes_it_timed(capi, n):
+    """The reported chunk is one that was timed: a listed length, or the one the
+    fused pass picks by itself (a listed length or the whole column)."""
+    ctx = capi.mhd_ctx_create(emf=1)
+    try:
+        p = to_patch(_moving(n, 2, 3, 0.3), n, 2, DX, dtype="f32")
+        d = torch.full((1,), 1e-3, dtype=torch.float64, device="cuda")
+        for _ in range(3):
+            choice, chunk, _ms = capi.mhd_autotune_advance(ctx, [p.desc()], d.data_ptr(), reps=1)
+            top = n[2] + 2
+            lengths = (2, 3, 4, 5, 6, 8, 10, 12, 14, 16, 20, 24, 28, 33, 40, 48, 66, 88, 130)
+            if choice <= -3:
+                assert chunk in {min(c, top) for c in lengths}, (choice, chunk)
+    finally:
+        capi.mhd_ctx_destroy(ctx)
