@@ -96,7 +96,7 @@ typedef struct {
   int32_t fp64_contract; /* MHD_F64 advance: 0 the parity build (no fused
                         multiply-add; every operation rounded as written, in
                         the oracle's order), 1 the build with multiply-adds
-                        fused (about 1.25x faster; differs from 0 by rounding) */
+                        fused (about 1.45x faster; differs from 0 by rounding) */
   int32_t advance_kernel; /* 0: the context's choice (what mhd_autotune_advance
                         measured fastest; before that the fused pass for
                         MHD_F32 calls of mhd_patch_advance without captures

@@ -113,7 +113,7 @@ __device__ __forceinline__ int flag_side(float a, float b, float c, float da, fl
 // and are decided at the end by the FP64 expressions, so the flags are those
 // of FP64.  (Seven FP64 pressures per cell took 230 FP64 instructions and
 // bound the kernel to the FP64 pipe.)  Measured on 200 patches of 8^3-64^3
-// cells (4.0 M cells, FP32): 2,300 -> 88 us; a first version with a fixed
+// cells (4.0 M cells, FP32): 2,300 -> 91 us; a first version with a fixed
 // tile, its rim computed by a third of the threads and the FP64 decision in
 // the loop took 138 us.
 template <typename R>
